@@ -17,52 +17,11 @@
 // J_el = -Hessian of the elastic energy is symmetric, so J_el m is the
 // directional derivative of the forces along m: k_tet_jvp runs the force
 // evaluation of mr.cuh on dual numbers. The forces are linear in
-// (mu_1, mu_2, kappa), so m . df/d(mu, kappa, w) comes from the forces at unit
-// moduli (k_param_vjp), reduced in double.
+// (mu_1, mu_2, kappa), so m . df/d(mu, kappa, w) comes from the rates of the
+// unit-modulus energies along m (mr_energy_rates), summed to 48 bits or more.
 #include "mr.cuh"
 
 namespace cf {
-
-// ---------------------------------------------------------------- JVP
-// Corner tangents d f / d eps of f(u + eps v) into m.fc.
-__global__ void __launch_bounds__(128) k_tet_jvp(MeshView m, const float4 *__restrict__ u,
-                                                 const float4 *__restrict__ v) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= m.T) return;
-    const int4 a4 = __ldg(m.tet + t);
-    float Bm[3][3];
-    load_B(m, t, Bm);
-    float H[3][3], dH[3][3];
-    tet_grad(__ldg(u + a4.x), __ldg(u + a4.y), __ldg(u + a4.z), __ldg(u + a4.w), Bm, H);
-    tet_grad(__ldg(v + a4.x), __ldg(v + a4.y), __ldg(v + a4.z), __ldg(v + a4.w), Bm, dH);
-    Dual Hd[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Hd[i][j] = Dual(H[i][j], dH[i][j]);
-    const float4 mat = __ldg(m.mat + mat_slot(m, t));
-    InvT<Dual> inv;
-    Dual P[3][3];
-    mr_stress(Hd, mat.x, mat.y, mat.z, inv, P);
-    float dP[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) dP[i][j] = P[i][j].d;
-    float f[4][3];
-    corner_forces(dP, Bm, __ldg(m.V0 + t), f);
-#pragma unroll
-    for (int a = 0; a < 4; ++a) m.fc[a * m.T + t] = make_float4(f[a][0], f[a][1], f[a][2], 0.f);
-}
-
-cudaError_t launch_force_jvp(const MeshView &m, const float4 *u, const float4 *v, float4 *out, unsigned *err,
-                             cudaStream_t s) {
-    if (m.T == 0) return cudaSuccess;
-    k_tet_jvp<<<(m.T + 127) / 128, 128, 0, s>>>(m, u, v);
-    MeshView g = m;
-    g.fv = out;
-    return launch_gather_spread(g, u, nullptr, nullptr, err, s);
-}
 
 // ---------------------------------------------------------------- parameters
 // Sum of `val` over the lanes of a warp that share cell c, added into
@@ -80,49 +39,137 @@ __device__ __forceinline__ void warp_cell_add(int c, double val, double *dst, in
     }
 }
 
-// lambda . df/d(mu, kappa, w) per cell, times `scale`, added into grad[3 c + .].
-__global__ void __launch_bounds__(128) k_param_vjp(MeshView m, const float4 *__restrict__ u,
+// From the sums G = lambda . df/d(mu1, mu2, kappa) of a cell, with
+// mu1 = w mu and mu2 = (1 - w) mu: its derivative with respect to mu (k = 0),
+// w (k = 1) or kappa (k = 2), times scale.
+__device__ __forceinline__ double moduli_rate(int k, double G0, double G1, double Gk, float4 mat, double scale) {
+    const double mu = (double)mat.x + (double)mat.y, w = (double)mat.w;
+    return scale * (k == 0 ? w * G0 + (1.0 - w) * G1 : k == 1 ? mu * (G0 - G1) : Gk);
+}
+
+// Add one tet per thread, g = lambda . df/d(mu1, mu2, kappa) of cell c (c < 0:
+// none), to its cell's gradient. Every thread of the block calls. Where the
+// block has one cell (the common case: a cell's tets are contiguous) its
+// threads are summed first, as float pairs (Sum2), and one goes on in FP64:
+// one addition per warp to a single cell's three sums took 35 us for 201 k tets
+// (6 k additions to the same address).
+constexpr int kVjpBlock = 128;
+
+__device__ __forceinline__ void block_add_moduli(const MeshView &m, int c, const float (&g)[3], double scale,
+                                                 double *grad) {
+    constexpr int kWarps = kVjpBlock / 32;
+    __shared__ Sum2 part[3][kWarps];
+    __shared__ int c0;
+    if (threadIdx.x == 0) c0 = c;  // the block's first tet: no later one has an element if it has none
+    __syncthreads();
+    if (__syncthreads_and(c == c0 || c < 0)) {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            Sum2 a;
+            a.hi = c < 0 ? 0.f : g[k];
+            warp_sum(a);
+            if (lane == 0) part[k][threadIdx.x >> 5] = a;
+        }
+        __syncthreads();
+        if (threadIdx.x >= 32 || c0 < 0) return;
+        Sum2 a;  // lane k: sum k over the warps
+        if (lane < 3)
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                a.add(part[lane][w].hi);
+                a.lo = __fadd_rn(a.lo, part[lane][w].lo);
+            }
+        const double G = a.value(), G0 = __shfl_sync(0xffffffffu, G, 0), G1 = __shfl_sync(0xffffffffu, G, 1);
+        if (lane < 3) atomicAdd(grad + 3 * c0 + (lane == 0 ? 0 : lane == 1 ? 2 : 1), moduli_rate(lane, G0, G1, G, __ldg(m.mat + c0), scale));
+    } else if (c >= 0) {
+        const float4 mat = __ldg(m.mat + c);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            atomicAdd(grad + 3 * c + (k == 0 ? 0 : k == 1 ? 2 : 1), moduli_rate(k, (double)g[0], (double)g[1], (double)g[2], mat, scale));
+    }
+}
+
+// lambda . df/d(mu, kappa, w) per cell, times `scale`, added into grad[3 c + .]:
+// the rates of the unit-modulus energies along lambda's gradient
+// (mr_energy_rates). Three stresses and 36 FP64 products per tet in its place
+// were bound by FP64: 201 k tets 53 us, now 9.9; 20 k tets 12.2 us, now 5.9.
+__global__ void __launch_bounds__(kVjpBlock) k_param_vjp(MeshView m, const float4 *__restrict__ u,
                                                    const float4 *__restrict__ lam, double scale, double *grad) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     int c = -1;
-    double dmu = 0.0, dkappa = 0.0, dw = 0.0;
+    float g[3] = {0.f, 0.f, 0.f};
     if (t < m.T) {
         const int4 a4 = __ldg(m.tet + t);
         float Bm[3][3];
         load_B(m, t, Bm);
-        float H[3][3];
+        float H[3][3], dH[3][3];
         tet_grad(__ldg(u + a4.x), __ldg(u + a4.y), __ldg(u + a4.z), __ldg(u + a4.w), Bm, H);
-        const float4 l[4] = {__ldg(lam + a4.x), __ldg(lam + a4.y), __ldg(lam + a4.z), __ldg(lam + a4.w)};
+        tet_grad(__ldg(lam + a4.x), __ldg(lam + a4.y), __ldg(lam + a4.z), __ldg(lam + a4.w), Bm, dH);
+        InvT<float> inv;
+        invariants_t(H, inv);
+        mr_energy_rates(H, dH, inv, g);
         const float V0 = __ldg(m.V0 + t);
-        double g[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {  // unit mu1, unit mu2, unit kappa
-            InvT<float> inv;
-            float P[3][3], f[4][3];
-            mr_stress(H, k == 0 ? 1.f : 0.f, k == 1 ? 1.f : 0.f, k == 2 ? 1.f : 0.f, inv, P);
-            corner_forces(P, Bm, V0, f);
-            double s = 0.0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) s += (double)l[a].x * f[a][0] + (double)l[a].y * f[a][1] + (double)l[a].z * f[a][2];
-            g[k] = s;
-        }
+        for (int k = 0; k < 3; ++k) g[k] *= -V0;
         c = __ldg(m.tcell + t);
-        const float4 mat = __ldg(m.mat + c);  // mu1, mu2, kappa, w
-        const double mu = (double)mat.x + (double)mat.y, w = (double)mat.w;
-        dmu = scale * (w * g[0] + (1.0 - w) * g[1]);
-        dkappa = scale * g[2];
-        dw = scale * mu * (g[0] - g[1]);
     }
-    warp_cell_add(c, dmu, grad, 3);
-    warp_cell_add(c, dkappa, grad + 1, 3);
-    warp_cell_add(c, dw, grad + 2, 3);
+    block_add_moduli(m, c, g, scale, grad);
 }
 
 cudaError_t launch_param_vjp(const MeshView &m, const float4 *u, const float4 *lam, double scale, double *grad,
                              cudaStream_t s) {
     if (m.T == 0) return cudaSuccess;
-    k_param_vjp<<<(m.T + 127) / 128, 128, 0, s>>>(m, u, lam, scale, grad);
+    k_param_vjp<<<(m.T + kVjpBlock - 1) / kVjpBlock, kVjpBlock, 0, s>>>(m, u, lam, scale, grad);
     return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------- JVP
+// Corner tangents d f / d eps of f(u + eps v) into m.fc. GRAD: the same
+// evaluation also adds v . df/d(mu, kappa, w), times `scale`, to grad: the
+// reverse step needs both along the same direction (528 k tets: 31 us, where
+// two launches took 20 + 126 us). Bound by its ~900 FP32 operations a tet.
+template <bool GRAD>
+__global__ void __launch_bounds__(GRAD ? kVjpBlock : 128) k_tet_jvp(MeshView m, const float4 *__restrict__ u,
+                                                 const float4 *__restrict__ v, double scale, double *grad) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (!GRAD && t >= m.T) return;
+    int c = -1;
+    float g[3] = {0.f, 0.f, 0.f};
+    if (t < m.T) {
+        const int4 a4 = __ldg(m.tet + t);
+        float Bm[3][3];
+        load_B(m, t, Bm);
+        float H[3][3], dH[3][3];
+        tet_grad(__ldg(u + a4.x), __ldg(u + a4.y), __ldg(u + a4.z), __ldg(u + a4.w), Bm, H);
+        tet_grad(__ldg(v + a4.x), __ldg(v + a4.y), __ldg(v + a4.z), __ldg(v + a4.w), Bm, dH);
+        const float4 mat = __ldg(m.mat + mat_slot(m, t));
+        const float V0 = __ldg(m.V0 + t);
+        float f[4][3];
+        InvT<float> inv;
+        tet_tangent(H, dH, mat, Bm, V0, inv, f);
+        if (GRAD) {
+            mr_energy_rates(H, dH, inv, g);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) g[k] *= -V0;
+            c = __ldg(m.tcell + t);
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) m.fc[a * m.T + t] = make_float4(f[a][0], f[a][1], f[a][2], 0.f);
+    }
+    if (GRAD) block_add_moduli(m, c, g, scale, grad);
+}
+
+cudaError_t launch_force_jvp(const MeshView &m, const float4 *u, const float4 *v, float4 *out, unsigned *err,
+                             cudaStream_t s, double scale, double *grad) {
+    if (m.T == 0) return cudaSuccess;
+    if (grad)
+        k_tet_jvp<true><<<(m.T + kVjpBlock - 1) / kVjpBlock, kVjpBlock, 0, s>>>(m, u, v, scale, grad);
+    else
+        k_tet_jvp<false><<<(m.T + 127) / 128, 128, 0, s>>>(m, u, v, 0.0, nullptr);
+    MeshView g = m;
+    g.fv = out;
+    return launch_gather_spread(g, u, nullptr, nullptr, err, s);
 }
 
 // ---------------------------------------------------------------- plates
@@ -204,20 +251,23 @@ __global__ void k_adj_m(int n, const float4 *__restrict__ ly, const float4 *__re
 }
 
 // lambda_y <- lambda_y + dt (J_el m + J_plate m), lambda_v <- c m at positions
-// u, with J_el m given (jv) and J_plate = diag(0, 0, -k) on penetrating
+// u, and m = dt lambda_y + lambda_v of the step before, with J_el m given (jv) and J_plate = diag(0, 0, -k) on penetrating
 // vertices.
 __global__ void k_adj_step(MeshView m, const float4 *__restrict__ u, const float4 *__restrict__ jv,
-                           const float4 *__restrict__ mvec, float4 *ly, float4 *lv, float dt, float c, float kp,
+                           float4 *mvec, float4 *ly, float4 *lv, float dt, float c, float kp,
                            const float *__restrict__ zlo, const float *__restrict__ zhi) {
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= m.V) return;
     const float4 xr = __ldg(m.xr + v);
     const PlateZ pz = plates_of(m, __float_as_int(xr.w), zlo, zhi);
     const float z = xr.z + __ldg(u + v).z;
-    const float4 l = ly[v], j = __ldg(jv + v), mm = __ldg(mvec + v);
+    const float4 l = ly[v], j = __ldg(jv + v), mm = mvec[v];
     const float jz = (z < pz.lo || z > pz.hi) ? -kp * mm.z : 0.f;
-    ly[v] = make_float4(l.x + dt * j.x, l.y + dt * j.y, l.z + dt * (j.z + jz), 0.f);
-    lv[v] = make_float4(c * mm.x, c * mm.y, c * mm.z, 0.f);
+    const float4 a = make_float4(l.x + dt * j.x, l.y + dt * j.y, l.z + dt * (j.z + jz), 0.f);
+    const float4 b = make_float4(c * mm.x, c * mm.y, c * mm.z, 0.f);
+    ly[v] = a;
+    lv[v] = b;
+    mvec[v] = make_float4(fmaf(dt, a.x, b.x), fmaf(dt, a.y, b.y), fmaf(dt, a.z, b.z), 0.f);
 }
 
 cudaError_t launch_adj_seed(const MeshView &m, const float4 *u, float kp, const float *zlo, const float *zhi,
@@ -232,7 +282,7 @@ cudaError_t launch_adj_m(int n, const float4 *ly, const float4 *lv, float dt, fl
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_step(const MeshView &m, const float4 *u, const float4 *jv, const float4 *mvec, float4 *ly,
+cudaError_t launch_adj_step(const MeshView &m, const float4 *u, const float4 *jv, float4 *mvec, float4 *ly,
                             float4 *lv, float dt, float c, float kp, const float *zlo, const float *zhi,
                             cudaStream_t s) {
     if (m.V == 0) return cudaSuccess;

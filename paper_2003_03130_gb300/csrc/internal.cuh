@@ -443,9 +443,10 @@ cudaError_t launch_interp_advect(const MeshView &m, const float4 *vel, const Lbm
                                  float4 *u_next, unsigned *err, cudaStream_t s, int block = 0,
                                  const RegionSlot &mark = RegionSlot{nullptr}, int form = 0);
 // Compression between plates and the adjoint (csrc/adjoint.cu).
-// out = J_el v at displacements u (vertex sums of the corner tangents; uses m.fc).
+// out = J_el v at displacements u (vertex sums of the corner tangents; uses m.fc);
+// with grad not null also grad[3 c + (0, 1, 2)] += scale * v . df/d(mu, kappa, w).
 cudaError_t launch_force_jvp(const MeshView &m, const float4 *u, const float4 *v, float4 *out, unsigned *err,
-                             cudaStream_t s);
+                             cudaStream_t s, double scale = 0.0, double *grad = nullptr);
 // grad[3 c + (0, 1, 2)] += scale * lambda . df/d(mu, kappa, w) per cell (double).
 cudaError_t launch_param_vjp(const MeshView &m, const float4 *u, const float4 *lam, double scale, double *grad,
                              cudaStream_t s);
@@ -457,7 +458,8 @@ cudaError_t launch_plate_force(const MeshView &m, const float4 *u, float kp, con
 cudaError_t launch_adj_seed(const MeshView &m, const float4 *u, float kp, const float *zlo, const float *zhi,
                             const double *dF, float4 *lam, cudaStream_t s);
 cudaError_t launch_adj_m(int n, const float4 *ly, const float4 *lv, float dt, float4 *mvec, cudaStream_t s);
-cudaError_t launch_adj_step(const MeshView &m, const float4 *u, const float4 *jv, const float4 *mvec, float4 *ly,
+// One reverse step; mvec holds m of this step on entry, of the step before on return.
+cudaError_t launch_adj_step(const MeshView &m, const float4 *u, const float4 *jv, float4 *mvec, float4 *ly,
                             float4 *lv, float dt, float c, float kp, const float *zlo, const float *zhi,
                             cudaStream_t s);
 cudaError_t launch_pack3(const double *in, int n, float4 *out, cudaStream_t s);

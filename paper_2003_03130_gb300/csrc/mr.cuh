@@ -140,6 +140,68 @@ __device__ __forceinline__ void mr_stress(const S (&H)[3][3], float mu1, float m
     mr_stress_inv(H, mu1, mu2, kappa, v, P);
 }
 
+// Rates of the three unit-modulus energies of one tet along dH: g = d/d eps of
+// (I - 3)/2, (K - 3)/2 and (J - 1)^2/2 at H + eps dH, so that a direction
+// lambda of the vertices with dH its gradient has lambda . f = -V0 g . (mu1,
+// mu2, kappa). One contraction per modulus takes the place of a stress and
+// twelve force components per modulus. With de = 2 (tr dH + H:dH) and
+// dj = tr dH + dj2, dj2 = t tr dH - tr(H dH) + cof(H):dH, the O(|dH|) parts
+// of de - 2 dj cancel by hand (J de - 2 dj = 2 (H:dH - dj2) + j de, and twice
+// that for K), so every term left is O(|H| |dH|), as in the stress:
+//   d(I) = s/J [J de - 2/3 (3 + e) dj],  s = J^-2/3,
+//   d(K) = s^2/J [J dK' - 4/3 K' dj],    K' = 3 + 2e + (e^2 - q)/2.
+__device__ __forceinline__ void mr_energy_rates(const float (&H)[3][3], const float (&dH)[3][3], const InvT<float> &v,
+                                                float (&g)[3]) {
+    const float dt = dH[0][0] + dH[1][1] + dH[2][2];
+    float hd = 0.f, hx = 0.f, eg = 0.f;  // H:dH, tr(H dH), E:(F^T dH)
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            hd += H[i][k] * dH[i][k];
+            hx += H[i][k] * dH[k][i];
+            eg += v.E[i][k] * (dH[i][k] + H[0][i] * dH[0][k] + H[1][i] * dH[1][k] + H[2][i] * dH[2][k]);
+        }
+    const float ddet = (H[1][1] * H[2][2] - H[1][2] * H[2][1]) * dH[0][0] + (H[1][2] * H[2][0] - H[1][0] * H[2][2]) * dH[0][1] +
+                       (H[1][0] * H[2][1] - H[1][1] * H[2][0]) * dH[0][2] + (H[0][2] * H[2][1] - H[0][1] * H[2][2]) * dH[1][0] +
+                       (H[0][0] * H[2][2] - H[0][2] * H[2][0]) * dH[1][1] + (H[0][1] * H[2][0] - H[0][0] * H[2][1]) * dH[1][2] +
+                       (H[0][1] * H[1][2] - H[0][2] * H[1][1]) * dH[2][0] + (H[0][2] * H[1][0] - H[0][0] * H[1][2]) * dH[2][1] +
+                       (H[0][0] * H[1][1] - H[0][1] * H[1][0]) * dH[2][2];
+    const float dj2 = v.t * dt - hx + ddet;
+    const float dj = dt + dj2, de = 2.f * (dt + hd), r = hd - dj2;
+    const float dk = v.e * de - 2.f * eg;  // dK' - 2 de, with dq = 4 E:(F^T dH)
+    const float k3 = 2.f * v.e + 0.5f * (v.e * v.e - v.q);
+    const float s = expf(-(2.f / 3.f) * v.L), iJ = 1.f / v.J;
+    g[0] = 0.5f * s * iJ * (2.f * r + v.j * de - (2.f / 3.f) * v.e * dj);
+    g[1] = 0.5f * s * s * iJ * (4.f * r + dk + v.j * (2.f * de + dk) - (4.f / 3.f) * k3 * dj);
+    g[2] = v.j * dj;
+}
+
+// A sum of floats kept as an unevaluated pair hi + lo: every addition is the
+// exact two-sum (D. E. Knuth, The Art of Computer Programming vol. 2, 4.2.2),
+// its error collected in lo, so the pair carries about 48 bits. FP64 units
+// are few on this GPU (about two additions per clock and SM); six FP32
+// additions per term are several times cheaper and as exact here.
+struct Sum2 {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)));
+        hi = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+// Sum of a pair over the lanes of a full warp (every lane ends with it).
+__device__ __forceinline__ void warp_sum(Sum2 &a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, a.hi, o), l = __shfl_xor_sync(0xffffffffu, a.lo, o);
+        a.add(h);
+        a.lo = __fadd_rn(a.lo, l);
+    }
+}
+
 // Nearly incompressible tets (kappa >= kStiffVolume (mu1 + mu2), Poisson
 // ratio 0.495 and above) take J - 1 in FP64. The volume term kappa (J - 1)
 // multiplies any rounding of J - 1 by kappa: under a nearly isochoric
@@ -220,6 +282,34 @@ __device__ __forceinline__ void tet_grad(const float4 &w0, const float4 &w1, con
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) H[i][j] = A[i][0] * Bm[0][j] + A[i][1] * Bm[1][j] + A[i][2] * Bm[2][j];
+}
+
+// Corner tangents along dH of a tet at H (the stress on dual numbers), and the
+// invariants at H.
+__device__ __forceinline__ void tet_tangent(const float (&H)[3][3], const float (&dH)[3][3], float4 mat,
+                                            const float (&Bm)[3][3], float V0, InvT<float> &inv, float (&f)[4][3]) {
+    Dual Hd[3][3], P[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) Hd[i][j] = Dual(H[i][j], dH[i][j]);
+    InvT<Dual> v;
+    mr_stress(Hd, mat.x, mat.y, mat.z, v, P);
+    float dP[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            dP[i][j] = P[i][j].d;
+            inv.E[i][j] = v.E[i][j].v;
+        }
+    corner_forces(dP, Bm, V0, f);
+    inv.t = v.t.v;
+    inv.e = v.e.v;
+    inv.q = v.q.v;
+    inv.j = v.j.v;
+    inv.J = v.J.v;
+    inv.L = v.L.v;
 }
 
 // Material slot of tet t.

@@ -230,6 +230,7 @@ cf_status cf_relax_adjoint(cf_ctx *c, const double *dF) {
     if (st != CF_OK) return st;
     CUDA_TRY(c, cudaMemcpyAsync(c->dF, dF, sizeof(double) * C, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, launch_adj_seed(m, c->ckpt[e.ck0 + e.nck - 1], e.kp, c->zlo, c->zhi, c->dF, c->lam, c->stream));
+    CUDA_TRY(c, launch_adj_m(c->V, c->lam, c->lamv, e.dt, c->mvec, c->stream));
     for (int j = e.nck - 2; j >= 0; --j) {
         const int s0 = j * kTapeStride, len = std::min(kTapeStride, e.n - s0);
         const size_t V = (size_t)c->V;
@@ -243,9 +244,7 @@ cf_status cf_relax_adjoint(cf_ctx *c, const double *dF) {
         }
         for (int i = len - 1; i >= 0; --i) {
             const float4 *y = c->seg + i * V;
-            CUDA_TRY(c, launch_adj_m(c->V, c->lam, c->lamv, e.dt, c->mvec, c->stream));
-            CUDA_TRY(c, launch_force_jvp(m, y, c->mvec, c->jv, c->d_err, c->stream));
-            CUDA_TRY(c, launch_param_vjp(m, y, c->mvec, (double)e.dt, c->grad, c->stream));
+            CUDA_TRY(c, launch_force_jvp(m, y, c->mvec, c->jv, c->d_err, c->stream, (double)e.dt, c->grad));
             CUDA_TRY(c, launch_adj_step(m, y, c->jv, c->mvec, c->lam, c->lamv, e.dt, e.c, e.kp, c->zlo, c->zhi,
                                         c->stream));
         }
