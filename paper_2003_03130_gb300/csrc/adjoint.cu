@@ -19,7 +19,7 @@
 // evaluation of mr.cuh on dual numbers. The forces are linear in
 // (mu_1, mu_2, kappa), so m . df/d(mu, kappa, w) comes from the rates of the
 // unit-modulus energies along m (mr_energy_rates), summed to 48 bits or more.
-#include "mr.cuh"
+#include "plate_ops.cuh"
 
 namespace cf {
 
@@ -37,14 +37,6 @@ __device__ __forceinline__ void warp_cell_add(int c, double val, double *dst, in
     } else if (c >= 0) {
         atomicAdd(dst + stride * c, val);
     }
-}
-
-// From the sums G = lambda . df/d(mu1, mu2, kappa) of a cell, with
-// mu1 = w mu and mu2 = (1 - w) mu: its derivative with respect to mu (k = 0),
-// w (k = 1) or kappa (k = 2), times scale.
-__device__ __forceinline__ double moduli_rate(int k, double G0, double G1, double Gk, float4 mat, double scale) {
-    const double mu = (double)mat.x + (double)mat.y, w = (double)mat.w;
-    return scale * (k == 0 ? w * G0 + (1.0 - w) * G1 : k == 1 ? mu * (G0 - G1) : Gk);
 }
 
 // Add one tet per thread, g = lambda . df/d(mu1, mu2, kappa) of cell c (c < 0:
@@ -81,12 +73,12 @@ __device__ __forceinline__ void block_add_moduli(const MeshView &m, int c, const
                 a.lo = __fadd_rn(a.lo, part[lane][w].lo);
             }
         const double G = a.value(), G0 = __shfl_sync(0xffffffffu, G, 0), G1 = __shfl_sync(0xffffffffu, G, 1);
-        if (lane < 3) atomicAdd(grad + 3 * c0 + (lane == 0 ? 0 : lane == 1 ? 2 : 1), moduli_rate(lane, G0, G1, G, __ldg(m.mat + c0), scale));
+        if (lane < 3) add_moduli_rate(lane, G0, G1, G, __ldg(m.mat + c0), scale, grad + 3 * c0);
     } else if (c >= 0) {
         const float4 mat = __ldg(m.mat + c);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-            atomicAdd(grad + 3 * c + (k == 0 ? 0 : k == 1 ? 2 : 1), moduli_rate(k, (double)g[0], (double)g[1], (double)g[2], mat, scale));
+            add_moduli_rate(k, (double)g[0], (double)g[1], (double)g[2], mat, scale, grad + 3 * c);
     }
 }
 
@@ -173,15 +165,6 @@ cudaError_t launch_force_jvp(const MeshView &m, const float4 *u, const float4 *v
 }
 
 // ---------------------------------------------------------------- plates
-struct PlateZ {
-    float lo, hi;  // plate heights relative to the cell's integer origin
-};
-
-__device__ __forceinline__ PlateZ plates_of(const MeshView &m, int c, const float *zlo, const float *zhi) {
-    const float oz = (float)__ldg(m.origin + 3 * c + 2);
-    return {__ldg(zlo + c) - oz, __ldg(zhi + c) - oz};
-}
-
 // v <- c v + dt (f_el + f_plate), y <- y + dt v from (u_in, v_in) into
 // (u_out, v_out); outputs may alias inputs.
 __global__ void k_plate_step(MeshView m, const float4 *u_in, const float4 *v_in, const float4 *__restrict__ fel,
@@ -191,11 +174,8 @@ __global__ void k_plate_step(MeshView m, const float4 *u_in, const float4 *v_in,
     if (v >= m.V) return;
     const float4 xr = __ldg(m.xr + v);
     const PlateZ pz = plates_of(m, __float_as_int(xr.w), zlo, zhi);
-    const float4 uu = u_in[v], vv = v_in[v], f = fel[v];
-    const float z = xr.z + uu.z;
-    const float fz = f.z + kp * fmaxf(pz.lo - z, 0.f) - kp * fmaxf(z - pz.hi, 0.f);
-    const float4 vn = make_float4(c * vv.x + dt * f.x, c * vv.y + dt * f.y, c * vv.z + dt * fz, 0.f);
-    const float4 un = make_float4(uu.x + dt * vn.x, uu.y + dt * vn.y, uu.z + dt * vn.z, 0.f);
+    float4 un, vn;
+    plate_move(u_in[v], v_in[v], fel[v], xr.z, pz, dt, c, kp, un, vn);
     if (!isfinite(un.x + un.y + un.z)) atomicOr(err, ERR_NONFINITE);
     u_out[v] = un;
     v_out[v] = vn;
@@ -261,13 +241,11 @@ __global__ void k_adj_step(MeshView m, const float4 *__restrict__ u, const float
     const float4 xr = __ldg(m.xr + v);
     const PlateZ pz = plates_of(m, __float_as_int(xr.w), zlo, zhi);
     const float z = xr.z + __ldg(u + v).z;
-    const float4 l = ly[v], j = __ldg(jv + v), mm = mvec[v];
-    const float jz = (z < pz.lo || z > pz.hi) ? -kp * mm.z : 0.f;
-    const float4 a = make_float4(l.x + dt * j.x, l.y + dt * j.y, l.z + dt * (j.z + jz), 0.f);
-    const float4 b = make_float4(c * mm.x, c * mm.y, c * mm.z, 0.f);
+    float4 a, b, mn;
+    adjoint_move(ly[v], __ldg(jv + v), mvec[v], z, pz, dt, c, kp, a, b, mn);
     ly[v] = a;
     lv[v] = b;
-    mvec[v] = make_float4(fmaf(dt, a.x, b.x), fmaf(dt, a.y, b.y), fmaf(dt, a.z, b.z), 0.f);
+    mvec[v] = mn;
 }
 
 cudaError_t launch_adj_seed(const MeshView &m, const float4 *u, float kp, const float *zlo, const float *zhi,

@@ -30,7 +30,7 @@ __device__ __forceinline__ void tet_load(const MeshView &m, const float4 *__rest
 
 // Corner forces of tet t from its inputs (Sec. 3.1): f^a = -V0 P B_a,
 // f^4 = -(f^1 + f^2 + f^3).
-__device__ __forceinline__ void tet_forces_store(const MeshView &m, const TetIn &in, unsigned *err, int t) {
+__device__ __forceinline__ void tet_corners(const MeshView &m, const TetIn &in, unsigned *err, int t, float (&f)[4][3]) {
     float H[3][3];
     tet_grad(in.w[0], in.w[1], in.w[2], in.w[3], in.Bm, H);
     InvT<float> v;
@@ -40,8 +40,12 @@ __device__ __forceinline__ void tet_forces_store(const MeshView &m, const TetIn 
         set_volume_change(v, (float)volume_change64(m.B64, m.T, t, in.w[0], in.w[1], in.w[2], in.w[3]));
     mr_stress_inv(H, in.mat.x, in.mat.y, in.mat.z, v, P);
     if (!(v.J > 0.f)) atomicOr(err, ERR_INVERTED);
-    float f[4][3];
     corner_forces(P, in.Bm, in.V0, f);
+}
+
+__device__ __forceinline__ void tet_forces_store(const MeshView &m, const TetIn &in, unsigned *err, int t) {
+    float f[4][3];
+    tet_corners(m, in, err, t, f);
 #pragma unroll
     for (int a = 0; a < 4; ++a) m.fc[a * m.T + t] = make_float4(f[a][0], f[a][1], f[a][2], 0.f);
 }

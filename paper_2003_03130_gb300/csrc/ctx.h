@@ -142,6 +142,15 @@ struct cf_ctx {
     float4 *seg = nullptr, *segv = nullptr;  // positions / velocities of one segment, (stride + 1) x V
     double *grad = nullptr, *gtmp = nullptr, *pforce = nullptr, *dF = nullptr;
     int adj_V = 0, adj_C = 0;
+    // on-chip relaxation (csrc/relax.cu): the plan of the current mesh, made
+    // by the first relaxation; plan_state 0: not tried, 1: made, 2: the mesh
+    // does not fit (general path)
+    int plan_state = 0;
+    RelaxPlan plan{};
+    RelaxPart *plan_parts = nullptr;
+    float4 *plan_rows = nullptr;
+    int *plan_list = nullptr;
+    uint4 *plan_inc = nullptr;
 
     int cur = 0;          // buffer parity of the next step
     long long tstep = 0;  // steps taken; tstep % 3 picks the region slots

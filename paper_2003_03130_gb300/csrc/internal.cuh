@@ -466,6 +466,40 @@ cudaError_t launch_adj_step(const MeshView &m, const float4 *u, const float4 *jv
                             cudaStream_t s);
 cudaError_t launch_pack3(const double *in, int n, float4 *out, cudaStream_t s);
 
+// Relaxation with a cell's state on chip (csrc/relax.cu): a cluster of `cs`
+// blocks per cell, block b holding the vertices [v0, v0 + nv) and every tet
+// that touches them.
+constexpr int kRelaxRound = 512;    // tets per block below which more blocks gain nothing
+constexpr int kRelaxStatic = 512;   // static shared memory of the step kernels, at most
+constexpr int kRelaxDegree = 32;    // incidences per vertex, at most
+struct RelaxPart {
+    int cell, cell_v0, cell_nv;  // the cell and its vertices
+    int v0, nv;                  // this part's vertices (global)
+    int t0, nt;                  // its tets in the plan's arrays
+};
+struct RelaxPlan {
+    int cs, nparts, NT;      // blocks per cell, parts, tets of all parts
+    int per_tet;             // tets have material slots of their own (MeshView::tmat)
+    size_t smem_step, smem_reverse;
+    const RelaxPart *parts;  // [nparts], cs per cell
+    const float4 *rows;      // [3][NT]
+    const int *list;         // [NT]
+    const uint4 *inc;        // [4][V] incidences, four lanes per vertex
+};
+size_t relax_smem(int cell_nv, int nt, bool reverse);
+cudaError_t prepare_relax(int smem_max);
+bool relax_fits(const RelaxPlan &pl);
+cudaError_t launch_relax_count(const MeshView &m, const int4 *cells, int ncells, int *counts, int *degree,
+                               cudaStream_t s);
+cudaError_t launch_relax_fill(const MeshView &m, const RelaxPart *parts, int nparts, int cs, const int4 *cells,
+                              float4 *rows, int NT, int *list, int *slot, uint4 *inc, cudaStream_t s);
+cudaError_t launch_relax_cells(const RelaxPlan &pl, const MeshView &m, const float4 *u_in, const float4 *v_in,
+                               float4 *u_out, float4 *v_out, float4 *ckpt, float4 *trail, float4 *fv, int n, float dt,
+                               float c, float kp, const float *zlo, const float *zhi, unsigned *err, cudaStream_t s);
+cudaError_t launch_relax_reverse(const RelaxPlan &pl, const MeshView &m, const float4 *y, float4 *ly, float4 *lv, int n,
+                                 float dt, float c, float kp, const float *zlo, const float *zhi, double *grad,
+                                 cudaStream_t s);
+
 cudaError_t launch_lbm_init(void *f, const LbmParams &p, cudaStream_t s);
 // rho and u(t) of every node after a step. u is u(t) as the near field
 // stored it (vel) on the last step's force region (bits, in the tiling of

@@ -55,6 +55,39 @@ __device__ __forceinline__ Dual m_rcp(Dual a) {
     return {r, -a.d * r * r};
 }
 
+// Sums of products with their roundings written out, so that every kernel
+// that evaluates a tet gets the same bits whatever surrounds it (left to the
+// compiler, which product of a sum is contracted depends on the context).
+__device__ __forceinline__ float m_dot3(float a, float b, float c, float d, float e, float f) {
+    return __fmaf_rn(e, f, __fmaf_rn(a, b, __fmul_rn(c, d)));
+}
+__device__ __forceinline__ Dual m_dot3(Dual a, Dual b, Dual c, Dual d, Dual e, Dual f) { return a * b + c * d + e * f; }
+__device__ __forceinline__ float m_cross(float a, float b, float c, float d) {  // a b - c d
+    return __fmaf_rn(a, b, -__fmul_rn(c, d));
+}
+__device__ __forceinline__ Dual m_cross(Dual a, Dual b, Dual c, Dual d) { return a * b - c * d; }
+// tr H^2 in row order; (1,2)(2,1) is rounded before it is added
+__device__ __forceinline__ float m_trace_sq(const float (&h)[3][3]) {
+    float s = __fmul_rn(h[0][0], h[0][0]);
+    s = __fmaf_rn(h[0][1], h[1][0], s);
+    s = __fmaf_rn(h[0][2], h[2][0], s);
+    s = __fmaf_rn(h[1][0], h[0][1], s);
+    s = __fmaf_rn(h[1][1], h[1][1], s);
+    const float q = __fmul_rn(h[1][2], h[2][1]);
+    s = __fadd_rn(s, q);
+    s = __fmaf_rn(h[2][0], h[0][2], s);
+    s = __fadd_rn(s, q);
+    return __fmaf_rn(h[2][2], h[2][2], s);
+}
+__device__ __forceinline__ Dual m_trace_sq(const Dual (&h)[3][3]) {
+    Dual s = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s = s + h[i][k] * h[k][i];
+    return s;
+}
+
 // ---------------------------------------------------------------- stress
 template <class S>
 struct InvT {
@@ -62,8 +95,12 @@ struct InvT {
     S E[3][3];
 };
 
-template <class S>
-__device__ __forceinline__ S det3t(const S (&h)[3][3]) {
+__device__ __forceinline__ float det3t(const float (&h)[3][3]) {
+    const float A = m_cross(h[1][1], h[2][2], h[1][2], h[2][1]), B = m_cross(h[1][0], h[2][2], h[1][2], h[2][0]),
+                C = m_cross(h[1][0], h[2][1], h[1][1], h[2][0]);
+    return __fmaf_rn(h[0][2], C, m_cross(h[0][0], A, h[0][1], B));
+}
+__device__ __forceinline__ Dual det3t(const Dual (&h)[3][3]) {
     return h[0][0] * (h[1][1] * h[2][2] - h[1][2] * h[2][1]) - h[0][1] * (h[1][0] * h[2][2] - h[1][2] * h[2][0]) +
            h[0][2] * (h[1][0] * h[2][1] - h[1][1] * h[2][0]);
 }
@@ -71,14 +108,12 @@ __device__ __forceinline__ S det3t(const S (&h)[3][3]) {
 template <class S>
 __device__ __forceinline__ void invariants_t(const S (&H)[3][3], InvT<S> &v) {
     v.t = H[0][0] + H[1][1] + H[2][2];
-    S trH2 = 0.f, hh = 0.f;
+    const S trH2 = m_trace_sq(H);
+    S hh = 0.f;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            trH2 = trH2 + H[i][k] * H[k][i];
-            hh = hh + H[i][k] * H[i][k];
-        }
+        for (int k = 0; k < 3; ++k) hh = hh + H[i][k] * H[i][k];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
@@ -112,20 +147,20 @@ __device__ __forceinline__ void mr_stress_inv(const S (&H)[3][3], float mu1, flo
     const S sigma = mu1 * s * (3.f * v.j - v.e) * iJ3 +
                     mu2 * s2 * (6.f * v.j - v.e + 3.f * v.j * v.e - v.e * v.e + v.q) * iJ3 + kappa * v.j;
     S cofH[3][3];
-    cofH[0][0] = H[1][1] * H[2][2] - H[1][2] * H[2][1];
-    cofH[0][1] = H[1][2] * H[2][0] - H[1][0] * H[2][2];
-    cofH[0][2] = H[1][0] * H[2][1] - H[1][1] * H[2][0];
-    cofH[1][0] = H[0][2] * H[2][1] - H[0][1] * H[2][2];
-    cofH[1][1] = H[0][0] * H[2][2] - H[0][2] * H[2][0];
-    cofH[1][2] = H[0][1] * H[2][0] - H[0][0] * H[2][1];
-    cofH[2][0] = H[0][1] * H[1][2] - H[0][2] * H[1][1];
-    cofH[2][1] = H[0][2] * H[1][0] - H[0][0] * H[1][2];
-    cofH[2][2] = H[0][0] * H[1][1] - H[0][1] * H[1][0];
+    cofH[0][0] = m_cross(H[1][1], H[2][2], H[1][2], H[2][1]);
+    cofH[0][1] = m_cross(H[1][2], H[2][0], H[1][0], H[2][2]);
+    cofH[0][2] = m_cross(H[1][0], H[2][1], H[1][1], H[2][0]);
+    cofH[1][0] = m_cross(H[0][2], H[2][1], H[0][1], H[2][2]);
+    cofH[1][1] = m_cross(H[0][0], H[2][2], H[0][2], H[2][0]);
+    cofH[1][2] = m_cross(H[0][1], H[2][0], H[0][0], H[2][1]);
+    cofH[2][0] = m_cross(H[0][1], H[1][2], H[0][2], H[1][1]);
+    cofH[2][1] = m_cross(H[0][2], H[1][0], H[0][0], H[1][2]);
+    cofH[2][2] = m_cross(H[0][0], H[1][1], H[0][1], H[1][0]);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
-            const S HE = H[i][0] * v.E[0][l] + H[i][1] * v.E[1][l] + H[i][2] * v.E[2][l];
+            const S HE = m_dot3(H[i][0], v.E[0][l], H[i][1], v.E[1][l], H[i][2], v.E[2][l]);
             S p = alpha * H[i][l] + beta * (cofH[i][l] - H[l][i]) + gamma * (H[i][l] + v.E[i][l] + HE);
             if (i == l) p = p + sigma + beta * v.t;
             P[i][l] = p;

@@ -11,11 +11,14 @@
 // walks it backwards with m = dt lambda_y + lambda_v:
 //   lambda_y <- lambda_y + dt (J_el + J_plate) m, lambda_v <- c m,
 // accumulating dt m . df/d(mu, kappa, w) per cell in double.
+#include <algorithm>
+
 #include "ctx.h"
 
 namespace {
 
 constexpr int kTapeStride = 50;
+constexpr int kRelaxSteps = 1000;  // steps of one launch, at most (some 10 ms)
 
 void free_adjoint(cf_ctx *c) {
     for (auto *p : c->ckpt) cudaFree(p);
@@ -37,6 +40,11 @@ void free_adjoint(cf_ctx *c) {
     dfree(c->dF);
     dfree(c->zlo);
     dfree(c->zhi);
+    dfree(c->plan_parts);
+    dfree(c->plan_rows);
+    dfree(c->plan_list);
+    dfree(c->plan_inc);
+    c->plan_state = 0;
     c->adj_V = c->adj_C = 0;
 }
 
@@ -77,6 +85,125 @@ cf_status ensure_adjoint(cf_ctx *c) {
         c->zhi_h.clear();
     }
     return CF_OK;
+}
+
+// The on-chip relaxation's plan for the current mesh, if it fits: cells cut
+// into `cs` blocks, the fewest that hold a part in shared memory; more, up to
+// eight, while every block still gets an SM of its own and a part has more
+// tets than threads. A mesh that does not fit, or no memory for the plan,
+// leaves the general path.
+cf_status make_plan(cf_ctx *c) {
+    if (c->plan_state) return CF_OK;
+    c->plan_state = 2;
+    const int C = (int)c->cells.size();
+    std::vector<int4> cells(C);
+    for (int k = 0; k < C; ++k) {
+        const CellInfo &ci = c->cells[k];
+        if (ci.nv > 0xffff) return CF_OK;
+        cells[k] = make_int4(ci.v_off, ci.nv, ci.t_off, ci.nt);
+    }
+    if (C > INT_MAX / 15) return CF_OK;
+    int smem = 0;
+    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+    if (smem <= kRelaxStatic || prepare_relax(smem) != cudaSuccess) {
+        cudaGetLastError();
+        return CF_OK;
+    }
+    const MeshView m = view(c);
+    int4 *d_cells = nullptr;
+    int *d_counts = nullptr, *d_slot = nullptr;
+    auto done = [&](cudaError_t e) {
+        dfree(d_cells);
+        dfree(d_counts);
+        dfree(d_slot);
+        if (c->plan_state != 1) {
+            dfree(c->plan_parts);
+            dfree(c->plan_rows);
+            dfree(c->plan_list);
+            dfree(c->plan_inc);
+        }
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // the general path needs none of it
+        return e == cudaSuccess || e == cudaErrorMemoryAllocation
+                   ? CF_OK
+                   : fail(c, CF_ECUDA, "relaxation plan: %s", cudaGetErrorString(e));
+    };
+#define TRY_P(expr)                               \
+    do {                                          \
+        const cudaError_t e_ = (expr);            \
+        if (e_ != cudaSuccess) return done(e_);   \
+    } while (0)
+    TRY_P(dalloc(&d_cells, C));
+    TRY_P(dalloc(&d_counts, 15 * (size_t)C + 1));
+    TRY_P(cudaMemcpyAsync(d_cells, cells.data(), sizeof(int4) * C, cudaMemcpyHostToDevice, c->stream));
+    TRY_P(launch_relax_count(m, d_cells, C, d_counts, d_counts + 15 * (size_t)C, c->stream));
+    std::vector<int> counts(15 * (size_t)C + 1);
+    TRY_P(cudaMemcpyAsync(counts.data(), d_counts, sizeof(int) * counts.size(), cudaMemcpyDeviceToHost, c->stream));
+    TRY_P(cudaStreamSynchronize(c->stream));
+    if (counts.back() > kRelaxDegree) return done(cudaSuccess);
+    auto largest = [&](int cs, bool &fits) {
+        int most = 0;
+        fits = true;
+        for (int k = 0; k < C; ++k)
+            for (int r = 0; r < cs; ++r) {
+                const int nt = counts[15 * (size_t)k + cs - 1 + r];
+                most = std::max(most, nt);
+                if (relax_smem(cells[k].y, nt, true) > (size_t)(smem - kRelaxStatic)) fits = false;
+            }
+        return most;
+    };
+    int cs = 1;
+    bool fits = false;
+    while (largest(cs, fits), !fits && cs < 8) cs *= 2;
+    if (!fits) return done(cudaSuccess);
+    while (cs < 8 && 2LL * cs * C <= c->sms && largest(cs, fits) > kRelaxRound) cs *= 2;
+    RelaxPlan pl{};
+    pl.cs = cs;
+    pl.nparts = cs * C;
+    std::vector<RelaxPart> parts(pl.nparts);
+    long long nt_all = 0;
+    for (int k = 0; k < C; ++k)
+        for (int r = 0; r < cs; ++r) {
+            RelaxPart &q = parts[(size_t)cs * k + r];
+            q.cell = k;
+            q.cell_v0 = cells[k].x;
+            q.cell_nv = cells[k].y;
+            q.v0 = cells[k].x + (int)((long long)cells[k].y * r / cs);
+            q.nv = cells[k].x + (int)((long long)cells[k].y * (r + 1) / cs) - q.v0;
+            q.t0 = (int)nt_all;
+            q.nt = counts[15 * (size_t)k + cs - 1 + r];
+            nt_all += q.nt;
+            pl.smem_step = std::max(pl.smem_step, relax_smem(q.cell_nv, q.nt, false));
+            pl.smem_reverse = std::max(pl.smem_reverse, relax_smem(q.cell_nv, q.nt, true));
+        }
+    if (nt_all > INT_MAX) return done(cudaSuccess);
+    pl.NT = (int)nt_all;
+    if (!relax_fits(pl)) return done(cudaSuccess);
+    TRY_P(dalloc(&c->plan_parts, parts.size()));
+    TRY_P(dalloc(&c->plan_rows, 3 * (size_t)pl.NT));
+    TRY_P(dalloc(&c->plan_list, pl.NT));
+    TRY_P(dalloc(&c->plan_inc, 4 * (size_t)c->V));
+    TRY_P(dalloc(&d_slot, (size_t)cs * c->T));
+    TRY_P(cudaMemcpyAsync(c->plan_parts, parts.data(), sizeof(RelaxPart) * parts.size(), cudaMemcpyHostToDevice,
+                          c->stream));
+    TRY_P(launch_relax_fill(m, c->plan_parts, pl.nparts, cs, d_cells, c->plan_rows, pl.NT, c->plan_list, d_slot,
+                            c->plan_inc, c->stream));
+    TRY_P(cudaStreamSynchronize(c->stream));  // the host vectors and the scratch go
+#undef TRY_P
+    pl.parts = c->plan_parts;
+    pl.rows = c->plan_rows;
+    pl.list = c->plan_list;
+    pl.inc = c->plan_inc;
+    c->plan = pl;
+    c->plan_state = 1;
+    return done(cudaSuccess);
+}
+
+// The plan if the mesh has one, with the materials' present form.
+const RelaxPlan *plan_of(cf_ctx *c) {
+    if (c->plan_state != 1) return nullptr;
+    c->plan.per_tet = 0;
+    for (const CellInfo &ci : c->cells) c->plan.per_tet |= ci.per_tet;
+    return &c->plan;
 }
 
 cf_status upload_plates(cf_ctx *c, const std::vector<float> &zlo, const std::vector<float> &zhi) {
@@ -167,7 +294,18 @@ cf_status cf_relax(cf_ctx *c, int32_t n, double dt, double damping, int32_t reco
             c->ckpt.push_back(p);
         }
     }
-    for (int k = 0; k < n; ++k) {
+    st = make_plan(c);
+    if (st != CF_OK) return st;
+    const RelaxPlan *pl = plan_of(c);
+    for (int k = 0; pl && k < n;) {  // on chip: a launch per checkpoint, or per kRelaxSteps
+        const int b = std::min(record ? kTapeStride : kRelaxSteps, n - k);
+        CUDA_TRY(c, launch_relax_cells(*pl, m, u, c->vel_r, u, c->vel_r,
+                                       record ? c->ckpt[e.ck0 + k / kTapeStride] : nullptr, nullptr,
+                                       k + b == n ? c->fv : nullptr, b, (float)dt, cd, c->k_plate, c->zlo, c->zhi,
+                                       c->d_err, c->stream));
+        k += b;
+    }
+    for (int k = 0; !pl && k < n; ++k) {
         if (record && k % kTapeStride == 0) {
             st = save_state(c, c->ckpt[e.ck0 + k / kTapeStride], u, c->vel_r);
             if (st != CF_OK) return st;
@@ -230,12 +368,24 @@ cf_status cf_relax_adjoint(cf_ctx *c, const double *dF) {
     if (st != CF_OK) return st;
     CUDA_TRY(c, cudaMemcpyAsync(c->dF, dF, sizeof(double) * C, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, launch_adj_seed(m, c->ckpt[e.ck0 + e.nck - 1], e.kp, c->zlo, c->zhi, c->dF, c->lam, c->stream));
-    CUDA_TRY(c, launch_adj_m(c->V, c->lam, c->lamv, e.dt, c->mvec, c->stream));
+    st = make_plan(c);
+    if (st != CF_OK) return st;
+    const RelaxPlan *pl = plan_of(c);
+    if (!pl) CUDA_TRY(c, launch_adj_m(c->V, c->lam, c->lamv, e.dt, c->mvec, c->stream));
     for (int j = e.nck - 2; j >= 0; --j) {
         const int s0 = j * kTapeStride, len = std::min(kTapeStride, e.n - s0);
         const size_t V = (size_t)c->V;
         const float4 *ck = c->ckpt[e.ck0 + j];
         CUDA_TRY(c, cudaMemcpyAsync(c->seg, ck, sizeof(float4) * V, cudaMemcpyDeviceToDevice, c->stream));
+        if (pl) {
+            if (len > 1)
+                CUDA_TRY(c, launch_relax_cells(*pl, m, ck, ck + V, c->seg + (size_t)(len - 1) * V, c->segv, nullptr,
+                                               c->seg, nullptr, len - 1, e.dt, e.c, e.kp, c->zlo, c->zhi, c->d_err,
+                                               c->stream));
+            CUDA_TRY(c, launch_relax_reverse(*pl, m, c->seg, c->lam, c->lamv, len, e.dt, e.c, e.kp, c->zlo, c->zhi,
+                                             c->grad, c->stream));
+            continue;
+        }
         CUDA_TRY(c, cudaMemcpyAsync(c->segv, ck + V, sizeof(float4) * V, cudaMemcpyDeviceToDevice, c->stream));
         for (int i = 0; i + 1 < len; ++i) {  // states of the segment's steps
             st = relax_step(c, m, c->seg + i * V, c->segv + i * V, c->seg + (i + 1) * V, c->segv + (i + 1) * V, e.dt,
