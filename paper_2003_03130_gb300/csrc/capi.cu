@@ -58,13 +58,17 @@ enum class Kind { First = 0, Mid = 1, Tail = 2, Fluid = 3, Single = 4 };
 // Region slots of step t (phase s = t % 3): the step's force region is slot
 // (s + 2) % 3 (filled by step t - 1, or from the current positions in the
 // first step of a call); the step fills the region of step t + 1 into slot
-// s. Three slots keep a slot from being cleared while a far-field kernel two
-// steps back may still read it.
+// s. The first step of a call empties the slots it fills, every near field the
+// one that the next step fills: the region of the step before this one, which
+// the far field that the near field waited for has read. Three slots keep a
+// slot from being cleared while a far-field kernel two steps back may still
+// read it.
 size_t tiles_of(const LbmParams &p) { return (size_t)p.ntx * p.nty * p.ntz; }
 
 RegionSlot slot_at(cf_ctx *c, int k) { return RegionSlot{c->region + c->region_stride * k}; }
 RegionSlot region_slot(cf_ctx *c, int s) { return slot_at(c, (s + 2) % 3); }
 RegionSlot accum_slot(cf_ctx *c, int s) { return slot_at(c, s); }
+RegionSlot next_slot(cf_ctx *c, int s) { return slot_at(c, (s + 1) % 3); }  // the step after's accum slot
 
 // Empty a slot: the bitset of the current tiling.
 cudaError_t clear_slot(const cf_ctx *c, const RegionSlot &r, cudaStream_t s) {
@@ -214,15 +218,14 @@ cf_status enqueue_steps(cf_ctx *c, Kind kind, int p0, int s0, int nsteps, cudaSt
         CUDA_TRY(c, launch_lbm_far(c->f[p], c->f[1 - p], sweep(c->lp, p), use.bits, c->seed + p, sh.far_spec, sf));
         CUDA_TRY(c, cudaEventRecord(ev_far[i], sf));
         if (!(first && i == 0)) {  // K5 of the previous step (parity 1-p), with mark_k5 marking acc
-            if (sh.mark_k5) CUDA_TRY(c, clear_slot(c, acc, sc));
             CUDA_TRY(c, launch_interp_advect(m, c->vel, c->lp, c->u[1 - p], c->u[p], c->d_err, sc, sh.interp_block,
                                              sh.mark_k5 ? acc : none, sh.interp_form));
         }
-        if (!sh.mark_k5) CUDA_TRY(c, clear_slot(c, acc, sc));
+        if (first && i == 0 && !sh.mark_k5) CUDA_TRY(c, clear_slot(c, acc, sc));
         CUDA_TRY(c, launch_chain_step(c, m, p, sh, acc, sc));
         if (i > 0) CUDA_TRY(c, cudaStreamWaitEvent(sc, ev_far[i - 1], 0));
         CUDA_TRY(c, launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c->lp, p), use.bits, c->vel,
-                                    sh.near_rows || !c->near_tiles_fit ? 0 : near_grid(c), c->seed + p, c->seed + 1 - p, sc));
+                                    sh.near_rows || !c->near_tiles_fit ? 0 : near_grid(c), c->seed + p, c->seed + 1 - p, next_slot(c, s).bits, sc));
         CUDA_TRY(c, cudaEventRecord(ev_near[i], sc));
     }
     if (kind == Kind::Single) {  // K5 of the last step, after its near field in sc order
@@ -962,19 +965,17 @@ cf_status timed_steps(cf_ctx *c, int n, const Shape &sh, double acc[5]) {
             const RegionSlot none{nullptr};
             if (cells && t == 0) {  // region of the first step (and, with mark_k5, the next): not timed
                 e = clear_slot(c, use, s);
-                if (e == cudaSuccess && sh.mark_k5) e = clear_slot(c, accm, s);
+                if (e == cudaSuccess) e = clear_slot(c, accm, s);
                 if (e == cudaSuccess) e = launch_mark_region(m, c->u[p], c->lp, use, sh.mark_k5 ? accm : none, s);
             }
-            if (cells && t > 0 && sh.mark_k5 && e == cudaSuccess) e = clear_slot(c, accm, s);
             cudaEventRecord(E[0], s);
             if (cells && t > 0 && e == cudaSuccess)
                 e = launch_interp_advect(m, c->vel, c->lp, c->u[1 - p], c->u[p], c->d_err, s, sh.interp_block,
                                          sh.mark_k5 ? accm : none, sh.interp_form);
             cudaEventRecord(E[1], s);
             if (cells && e == cudaSuccess) {
-                if (!sh.mark_k5) e = clear_slot(c, accm, s);
-                if (e == cudaSuccess && sh.fused) e = launch_chain_step(c, m, p, sh, accm, s);
-                if (e == cudaSuccess && !sh.fused)
+                if (sh.fused) e = launch_chain_step(c, m, p, sh, accm, s);
+                else
                     e = launch_tet_force(m, c->u[p], c->d_err, s, sh.tet_block, sh.tet_form,
                                          sh.mark_k5 ? nullptr : &c->lp, sh.mark_k5 ? nullptr : &accm);
             }
@@ -988,7 +989,8 @@ cf_status timed_steps(cf_ctx *c, int n, const Shape &sh, double acc[5]) {
             cudaEventRecord(E[4], s);
             if (cells && e == cudaSuccess)
                 e = launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c->lp, p), use.bits, c->vel,
-                                    sh.near_rows || !c->near_tiles_fit ? 0 : near_grid(c), c->seed + p, c->seed + 1 - p, s);
+                                    sh.near_rows || !c->near_tiles_fit ? 0 : near_grid(c), c->seed + p, c->seed + 1 - p,
+                                    next_slot(c, sph).bits, s);
             cudaEventRecord(E[5], s);
             c->cur ^= 1;
             c->tstep += 1;

@@ -421,9 +421,11 @@ cudaError_t launch_lbm_far(const void *fin, void *fout, const LbmParams &p, cons
                            const unsigned *seed, bool spec, cudaStream_t s);
 // blocks > 0: that many blocks stride over the region's tiles (the set bits
 // of its bitset); blocks <= 0: rows of 128 nodes over the whole lattice,
-// threads outside the region return at once.
+// threads outside the region return at once. clear: a region slot that the
+// launch empties.
 cudaError_t launch_lbm_near(const void *fin, void *fout, float4 *F, const LbmParams &p, const unsigned *bits,
-                            float4 *vel, int blocks, const unsigned *seed, unsigned *next_seed, cudaStream_t s);
+                            float4 *vel, int blocks, const unsigned *seed, unsigned *next_seed, unsigned *clear,
+                            cudaStream_t s);
 // Shared-memory opt-in of the list-form near field (its per-block running
 // counts of the region bitset; once per context, before any capture).
 cudaError_t prepare_near_field(long long max_words);

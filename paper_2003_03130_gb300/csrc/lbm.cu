@@ -560,6 +560,19 @@ __device__ __forceinline__ void lbm_pair(const T *__restrict__ fin, T *__restric
 // of a lattice that is swept to and fro.
 __device__ __forceinline__ int plane_of(const LbmParams &p, int z) { return p.back ? p.nz - 1 - z : z; }
 
+// The near field also empties the region slot of the step after next's
+// marking (nobody reads it any more: it was the region of the step before),
+// so that no memset stands in the chain of a step's kernels. Thread `i` of
+// `n` threads takes its share.
+__device__ __forceinline__ void clear_words(unsigned *w, int nwords, long long i, long long n) {
+    for (; i < nwords; i += n) w[i] = 0u;
+}
+
+__device__ __forceinline__ void clear_words_rows(unsigned *w, int nwords) {
+    const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
+    clear_words(w, nwords, b * blockDim.x + threadIdx.x, (long long)gridDim.x * gridDim.y * gridDim.z * blockDim.x);
+}
+
 // Whole lattice, no force field (fluid-only runs).
 template <class T>
 __global__ void __launch_bounds__(128) k_lbm(const T *__restrict__ fin, T *__restrict__ fout, LbmParams p,
@@ -618,8 +631,9 @@ template <class T, bool CS = true>
 __global__ void __launch_bounds__(128) k_lbm_near_rows(const T *__restrict__ fin, T *__restrict__ fout,
                                                        float4 *__restrict__ F, LbmParams p,
                                                        const unsigned *__restrict__ bits, float4 *__restrict__ vel,
-                                                       const unsigned *__restrict__ seed_in,
+                                                       const unsigned *__restrict__ seed_in, unsigned *clear, int nwords,
                                                        unsigned *__restrict__ seed_out) {
+    clear_words_rows(clear, nwords);
     const unsigned seed = *seed_in;
     if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *seed_out = seed + 1u;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -644,10 +658,11 @@ __global__ void __launch_bounds__(kTileBlock, 8) k_lbm_near(const T *__restrict_
                                                             float4 *__restrict__ F, LbmParams p,
                                                             const unsigned *__restrict__ bits, int nwords,
                                                             float4 *__restrict__ vel,
-                                                            const unsigned *__restrict__ seed_in,
+                                                            const unsigned *__restrict__ seed_in, unsigned *clear,
                                                             unsigned *__restrict__ seed_out) {
     extern __shared__ int before[];  // [nwords + 1]: set bits in the words before word j
     __shared__ int warp_sum[kTileBlock / 32];
+    clear_words(clear, nwords, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
     const unsigned seed = *seed_in;
     if ((blockIdx.x | threadIdx.x) == 0) *seed_out = seed + 1u;
     // running counts: thread i takes a contiguous chunk of words
@@ -735,8 +750,9 @@ template <class T>
 __global__ void __launch_bounds__(64) k_lbm_near_pairs(const T *__restrict__ fin, T *__restrict__ fout,
                                                        float4 *__restrict__ F, LbmParams p,
                                                        const unsigned *__restrict__ bits, float4 *__restrict__ vel,
-                                                       const unsigned *__restrict__ seed_in,
+                                                       const unsigned *__restrict__ seed_in, unsigned *clear, int nwords,
                                                        unsigned *__restrict__ seed_out) {
+    clear_words_rows(clear, nwords);
     const unsigned seed = *seed_in;
     if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *seed_out = seed + 1u;
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -860,7 +876,8 @@ static cudaError_t far_t(const void *fin, void *fout, const LbmParams &p, const 
 
 template <class T>
 static cudaError_t near_t(const void *fin, void *fout, float4 *F, const LbmParams &p, const unsigned *bits,
-                          float4 *vel, int blocks, const unsigned *seed, unsigned *next_seed, cudaStream_t s) {
+                          float4 *vel, int blocks, const unsigned *seed, unsigned *next_seed, unsigned *clear,
+                          cudaStream_t s) {
     const int nwords = (int)(((long long)p.ntx * p.nty * p.ntz + 31) / 32);
     const size_t smem = sizeof(int) * ((size_t)nwords + 1);
     if constexpr (std::is_same<T, float>::value) {
@@ -869,11 +886,11 @@ static cudaError_t near_t(const void *fin, void *fout, float4 *F, const LbmParam
                 const int bx = p.nx < 128 ? p.nx : 128;
                 dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
                 k_lbm_near_rows<T, false><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), F, p,
-                                                              bits, vel, seed, next_seed);
+                                                              bits, vel, seed, clear, nwords, next_seed);
             } else {
                 k_lbm_near<T, false><<<blocks, kTileBlock, smem, s>>>(static_cast<const T *>(fin),
                                                                       static_cast<T *>(fout), F, p, bits, nwords, vel,
-                                                                      seed, next_seed);
+                                                                      seed, clear, next_seed);
             }
             return cudaGetLastError();
         }
@@ -883,7 +900,7 @@ static cudaError_t near_t(const void *fin, void *fout, float4 *F, const LbmParam
             int bx;
             const dim3 grid = pair_grid(p, bx);
             k_lbm_near_pairs<T><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), F, p, bits,
-                                                     vel, seed, next_seed);
+                                                     vel, seed, clear, nwords, next_seed);
             return cudaGetLastError();
         }
     }
@@ -891,11 +908,11 @@ static cudaError_t near_t(const void *fin, void *fout, float4 *F, const LbmParam
         const int bx = p.nx < 128 ? p.nx : 128;
         dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
         k_lbm_near_rows<T><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), F, p, bits, vel,
-                                               seed, next_seed);
+                                               seed, clear, nwords, next_seed);
         return cudaGetLastError();
     }
     k_lbm_near<T><<<blocks, kTileBlock, smem, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), F, p, bits,
-                                                   nwords, vel, seed, next_seed);
+                                                   nwords, vel, seed, clear, next_seed);
     return cudaGetLastError();
 }
 
@@ -939,11 +956,12 @@ cudaError_t launch_lbm_far(const void *fin, void *fout, const LbmParams &p, cons
 }
 
 cudaError_t launch_lbm_near(const void *fin, void *fout, float4 *F, const LbmParams &p, const unsigned *bits,
-                            float4 *vel, int blocks, const unsigned *seed, unsigned *next_seed, cudaStream_t s) {
+                            float4 *vel, int blocks, const unsigned *seed, unsigned *next_seed, unsigned *clear,
+                            cudaStream_t s) {
     switch (p.fmt) {
-        case POP_F16: return near_t<__half>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, s);
-        case POP_BF16: return near_t<__nv_bfloat16>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, s);
-        default: return near_t<float>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, s);
+        case POP_F16: return near_t<__half>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, clear, s);
+        case POP_BF16: return near_t<__nv_bfloat16>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, clear, s);
+        default: return near_t<float>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, clear, s);
     }
 }
 
