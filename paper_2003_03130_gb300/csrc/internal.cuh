@@ -489,7 +489,7 @@ struct RelaxPlan {
     const int *list;         // [NT]
     const uint4 *inc;        // [4][V] incidences, four lanes per vertex
 };
-size_t relax_smem(int cell_nv, int nt, bool reverse);
+size_t relax_smem(int cell_nv, int nv, int nt, bool reverse);
 cudaError_t prepare_relax(int smem_max);
 bool relax_fits(const RelaxPlan &pl);
 cudaError_t launch_relax_count(const MeshView &m, const int4 *cells, int ncells, int *counts, int *degree,

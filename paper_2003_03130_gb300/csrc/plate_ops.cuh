@@ -17,13 +17,15 @@ __device__ __forceinline__ PlateZ plates_of(const MeshView &m, int c, const floa
 }
 
 // v <- c v + dt (f_el + f_plate), y <- y + dt v of a vertex at displacement uu,
-// velocity vv, with elastic force f and reference height zr.
+// velocity vv, with elastic force f and reference height zr; the roundings
+// written out, so that every path takes the same step bit for bit.
 __device__ __forceinline__ void plate_move(float4 uu, float4 vv, float4 f, float zr, PlateZ pz, float dt, float c,
                                            float kp, float4 &un, float4 &vn) {
-    const float z = zr + uu.z;
-    const float fz = f.z + kp * fmaxf(pz.lo - z, 0.f) - kp * fmaxf(z - pz.hi, 0.f);
-    vn = make_float4(c * vv.x + dt * f.x, c * vv.y + dt * f.y, c * vv.z + dt * fz, 0.f);
-    un = make_float4(uu.x + dt * vn.x, uu.y + dt * vn.y, uu.z + dt * vn.z, 0.f);
+    const float z = __fadd_rn(zr, uu.z);
+    const float fz = __fmaf_rn(-kp, fmaxf(z - pz.hi, 0.f), __fmaf_rn(kp, fmaxf(pz.lo - z, 0.f), f.z));
+    vn = make_float4(__fmaf_rn(c, vv.x, __fmul_rn(dt, f.x)), __fmaf_rn(c, vv.y, __fmul_rn(dt, f.y)),
+                     __fmaf_rn(c, vv.z, __fmul_rn(dt, fz)), 0.f);
+    un = make_float4(__fmaf_rn(dt, vn.x, uu.x), __fmaf_rn(dt, vn.y, uu.y), __fmaf_rn(dt, vn.z, uu.z), 0.f);
 }
 
 // lambda_y <- lambda_y + dt (J_el m + J_plate m), lambda_v <- c m of a vertex at

@@ -147,7 +147,7 @@ cf_status make_plan(cf_ctx *c) {
             for (int r = 0; r < cs; ++r) {
                 const int nt = counts[15 * (size_t)k + cs - 1 + r];
                 most = std::max(most, nt);
-                if (relax_smem(cells[k].y, nt, true) > (size_t)(smem - kRelaxStatic)) fits = false;
+                if (relax_smem(cells[k].y, cells[k].y, nt, true) > (size_t)(smem - kRelaxStatic)) fits = false;
             }
         return most;
     };
@@ -172,8 +172,8 @@ cf_status make_plan(cf_ctx *c) {
             q.t0 = (int)nt_all;
             q.nt = counts[15 * (size_t)k + cs - 1 + r];
             nt_all += q.nt;
-            pl.smem_step = std::max(pl.smem_step, relax_smem(q.cell_nv, q.nt, false));
-            pl.smem_reverse = std::max(pl.smem_reverse, relax_smem(q.cell_nv, q.nt, true));
+            pl.smem_step = std::max(pl.smem_step, relax_smem(q.cell_nv, q.nv, q.nt, false));
+            pl.smem_reverse = std::max(pl.smem_reverse, relax_smem(q.cell_nv, q.nv, q.nt, true));
         }
     if (nt_all > INT_MAX) return done(cudaSuccess);
     pl.NT = (int)nt_all;

@@ -18,15 +18,19 @@
 // per vertex, a fixed tree), and the tets run the same code, so the positions
 // are those of the general path (three launches a step, k_tet_force,
 // k_gather_spread, k_plate_step), bit for bit. That path stays for cells
-// that do not fit: shared memory holds 16 bytes per vertex of the cell and 36
-// per tet of a block (the reverse step 32 and 36), up to eight blocks a
+// that do not fit: shared memory holds 16 bytes per vertex of the cell, 16 more
+// per vertex and 36 per tet of a block (the reverse step 32 and 36), up to eight blocks a
 // cluster, 65,535 vertices a cell and 32 incidences a vertex.
 //
 // Bound by instruction issue (0.6 of the slots: ~400 instructions a tet, ~40
-// an incidence). 64 cells of 8.3 k tets (1,853 vertices) on 128 SMs: 19 us a
+// an incidence). 64 cells of 8.3 k tets (1,853 vertices) on 128 SMs: 17.5 us a
 // step, where the three launches took 29 (the corner forces cross L2 there, 64
 // bytes written and read per tet); a reverse step 36 us, 53 before. Two cells
-// of 1.2 k tets: 6 us a step of either kind, 15 and 25 before.
+// of 1.2 k tets: 5 to 6 us a step of either kind, 15 and 25 before. Velocities
+// stay in shared memory and the trail is stored a step late, since a barrier's
+// release waits for every store still on its way (19 -> 17.5 us). Measured and
+// not taken: every tet in one block only, corner forces read from the
+// neighbour through distributed shared memory (20.5 us).
 #include <climits>
 
 #include "cell_ops.cuh"
@@ -213,28 +217,39 @@ __device__ __forceinline__ void sum_incidences(const uint4 &e, const float *fc, 
 // n damped steps of all cells from (u_in, v_in) to (u_out, v_out), which may be
 // the same arrays. ckpt (may be null) receives the state before the first step
 // (displacements, then velocities); trail (may be null) the displacements
-// after every step, step i at trail + (i + 1) V; fv (may be null) the elastic
-// forces of the last step.
+// after every step but the last, step i at trail + (i + 1) V; fv (may be null) the elastic
+// forces of the last step. The last step's displacements go to u_out alone.
 __global__ void __launch_bounds__(kStepBlock, 1)
     k_relax_cells(RelaxPlan pl, MeshView m, const float4 *u_in, const float4 *v_in, float4 *u_out, float4 *v_out,
                   float4 *ckpt, float4 *trail, float4 *fv, int n, float dt, float c, float kp,
                   const float *__restrict__ zlo, const float *__restrict__ zhi, unsigned *err) {
-    extern __shared__ float4 su[];  // [vertices of the cell], then the corner forces
+    // [vertices of the cell] displacements, [own] velocities, the corner forces
+    extern __shared__ float4 su[];
     const cg::cluster_group cluster = cg::this_cluster();
     const RelaxPart p = pl.parts[blockIdx.x];
-    float *fc = reinterpret_cast<float *>(su + p.cell_nv);
+    float4 *sv = su + p.cell_nv;
+    float *fc = reinterpret_cast<float *>(sv + p.nv);
     const int lane = threadIdx.x & 3;
     const float4 cell_mat = __ldg(m.mat + p.cell);
     const bool by_index = pl.per_tet || needs_fp64_volume(m, cell_mat);
     const PlateZ pz = plates_of(m, p.cell, zlo, zhi);
     for (int j = threadIdx.x; j < p.cell_nv; j += kStepBlock) su[j] = u_in[p.cell_v0 + j];
-    if (ckpt)
-        for (int v = p.v0 + threadIdx.x; v < p.v0 + p.nv; v += kStepBlock) {
+    for (int j = threadIdx.x; j < p.nv; j += kStepBlock) {
+        const int v = p.v0 + j;
+        const float4 vel = v_in[v];
+        sv[j] = vel;
+        if (ckpt) {
             ckpt[v] = u_in[v];
-            ckpt[m.V + v] = v_in[v];
+            ckpt[m.V + v] = vel;
         }
+    }
     __syncthreads();
     for (int step = 0; step < n; ++step) {
+        // the displacements of the step before, here rather than where they
+        // are made: a store that is still on its way holds up a barrier's release
+        if (trail && step > 0)
+            for (int j = threadIdx.x; j < p.nv; j += kStepBlock)
+                trail[(size_t)step * m.V + p.v0 + j] = su[p.v0 - p.cell_v0 + j];
 #pragma unroll 1
         for (int i = threadIdx.x; i < p.nt; i += kStepBlock) {
             TetIn in;
@@ -251,14 +266,11 @@ __global__ void __launch_bounds__(kStepBlock, 1)
             for (int k = 0; k < 9; ++k) fc[9 * i + k] = f[k / 3][k % 3];
         }
         // first rows before the barrier, so that their latency hides under it
-        const float4 *vs = step == 0 ? v_in : v_out;
         uint4 e = make_uint4(~0u, ~0u, ~0u, ~0u);
-        float4 vv = make_float4(0.f, 0.f, 0.f, 0.f);
         float z0 = 0.f;
         auto fetch = [&](int j) {
             if (j < p.nv) {
                 e = __ldg(pl.inc + 4 * (size_t)(p.v0 + j) + lane);
-                vv = vs[p.v0 + j];
                 z0 = __ldg(m.xr + p.v0 + j).z;
             } else {
                 e = make_uint4(~0u, ~0u, ~0u, ~0u);
@@ -270,26 +282,24 @@ __global__ void __launch_bounds__(kStepBlock, 1)
         for (int j0 = 0; j0 == 0 || j0 < p.nv; j0 += kStepBlock / 4) {
             const int j = j0 + (threadIdx.x >> 2), v = p.v0 + j, local = v - p.cell_v0;
             const uint4 ee = e;
-            const float4 v_now = vv;
             const float zr = z0;
             if (j0 + kStepBlock / 4 < p.nv) fetch(j + kStepBlock / 4);
             float fx, fy, fz;
             sum_incidences(ee, fc, fx, fy, fz);
             const bool live = j < p.nv;
             float4 un = make_float4(0.f, 0.f, 0.f, 0.f), vn = un;
-            if (live) plate_move(su[local], v_now, make_float4(fx, fy, fz, 0.f), zr, pz, dt, c, kp, un, vn);
+            if (live) plate_move(su[local], sv[j], make_float4(fx, fy, fz, 0.f), zr, pz, dt, c, kp, un, vn);
             if (j0 == 0) cluster.barrier_wait();  // every block is done with the old displacements
             __syncwarp();                         // the four lanes have read theirs
             if (!live) continue;
             for (int r = lane; r < pl.cs; r += 4) *cluster.map_shared_rank(su + local, r) = un;
             if (lane == 0) {
                 if (!isfinite(fx + fy + fz) || !isfinite(un.x + un.y + un.z)) atomicOr(err, ERR_NONFINITE);
-                v_out[v] = vn;
-            } else if (lane == 1) {
-                if (trail) trail[(size_t)(step + 1) * m.V + v] = un;
-                if (step == n - 1) u_out[v] = un;
-            } else if (lane == 2 && fv && step == n - 1) {
-                fv[v] = make_float4(fx, fy, fz, 0.f);
+                sv[j] = vn;
+            } else if (step == n - 1) {
+                if (lane == 1) u_out[v] = un;
+                if (lane == 2) v_out[v] = vn;
+                if (lane == 3 && fv) fv[v] = make_float4(fx, fy, fz, 0.f);
             }
         }
         cluster.sync();  // the new displacements are everywhere
@@ -383,8 +393,8 @@ __global__ void __launch_bounds__(kReverseBlock, 1)
 }
 
 // ---------------------------------------------------------------- launchers
-size_t relax_smem(int cell_nv, int nt, bool reverse) {
-    return sizeof(float4) * (size_t)cell_nv * (reverse ? 2 : 1) + sizeof(float) * 9 * (size_t)nt;
+size_t relax_smem(int cell_nv, int nv, int nt, bool reverse) {
+    return sizeof(float4) * ((size_t)cell_nv * (reverse ? 2 : 1) + (reverse ? 0 : nv)) + sizeof(float) * 9 * (size_t)nt;
 }
 
 cudaError_t prepare_relax(int smem_max) {
