@@ -396,9 +396,9 @@ cf_status cf_create(cf_ctx **out, int device, void *cuda_stream) {
     const bool err_ok =
         c->err_mapped || (dalloc(&c->d_err, 1) == cudaSuccess && cudaMemset(c->d_err, 0, sizeof(unsigned)) == cudaSuccess &&
                           cudaMallocHost((void **)&c->h_err, sizeof(unsigned)) == cudaSuccess);
-    if (!err_ok || dalloc(&c->d_status, 1) != cudaSuccess || dalloc(&c->taylor_out, 10) != cudaSuccess ||
-        dalloc(&c->seed, 2) != cudaSuccess || cudaMemset(c->seed, 0, 2 * sizeof(unsigned)) != cudaSuccess ||
-        dalloc(&c->energy_out, 1) != cudaSuccess) {
+    if (!err_ok || dalloc(&c->d_status, 1) != cudaSuccess || dalloc(&c->seed, 2) != cudaSuccess ||
+        cudaMemset(c->seed, 0, 2 * sizeof(unsigned)) != cudaSuccess ||
+        cudaHostAlloc((void **)&c->result, 10 * sizeof(double), cudaHostAllocMapped) != cudaSuccess) {
         cf_destroy(c);
         return CF_ENOMEM;
     }
@@ -446,10 +446,9 @@ void cf_destroy(cf_ctx *c) {
     dfree(c->csr_idx);
     dfree(c->csr_cursor);
     dfree(c->energy_partial);
-    dfree(c->energy_out);
     dfree(c->stage);
     dfree(c->taylor_partial);
-    dfree(c->taylor_out);
+    if (c->result) cudaFreeHost(c->result);
     cf_free_adjoint(c);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -1309,20 +1308,22 @@ cf_status cf_get_energy(cf_ctx *c, int32_t id, double *out) {
     const CellInfo *ci = cell_of(c, id);
     if (!ci || !out) return fail(c, CF_EINVAL, "unknown cell or null output");
     DeviceGuard dg(c->device);
-    CUDA_TRY(c, launch_energy(view(c), c->u[c->cur], ci->t_off, ci->t_off + ci->nt, c->energy_partial, c->energy_out,
+    CUDA_TRY(c, launch_energy(view(c), c->u[c->cur], ci->t_off, ci->t_off + ci->nt, c->energy_partial, c->result,
                               c->stream));
-    CUDA_TRY(c, cudaMemcpyAsync(out, c->energy_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    return wait_stream(c);
+    const cf_status s = wait_stream(c);
+    if (s == CF_OK) *out = c->result[0];
+    return s;
 }
 
 cf_status cf_get_taylor(cf_ctx *c, int32_t id, double *out) {
     const CellInfo *ci = cell_of(c, id);
     if (!ci || !out) return fail(c, CF_EINVAL, "unknown cell or null output");
     DeviceGuard dg(c->device);
-    CUDA_TRY(c, launch_taylor(view(c), c->u[c->cur], ci->t_off, ci->t_off + ci->nt, c->taylor_partial, c->taylor_out,
+    CUDA_TRY(c, launch_taylor(view(c), c->u[c->cur], ci->t_off, ci->t_off + ci->nt, c->taylor_partial, c->result,
                               c->stream));
-    CUDA_TRY(c, cudaMemcpyAsync(out, c->taylor_out, 10 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    return wait_stream(c);
+    const cf_status s = wait_stream(c);
+    if (s == CF_OK) std::memcpy(out, c->result, 10 * sizeof(double));
+    return s;
 }
 
 cf_status cf_get_cell_strain(cf_ctx *c, int32_t id, double d_ref, double *out) {
@@ -1333,12 +1334,11 @@ cf_status cf_get_cell_strain(cf_ctx *c, int32_t id, double d_ref, double *out) {
     unsigned *word = reinterpret_cast<unsigned *>(c->d_status);  // device scratch of the context: two words
     float4 *keep = reinterpret_cast<float4 *>(c->stage);          // and 24 bytes per vertex
     CUDA_TRY(c, launch_max_extent(view(c), c->u[c->cur], ci->v_off, ci->nv, keep, word, 4 * c->sms, c->stream));
-    unsigned bits = 0;
-    CUDA_TRY(c, cudaMemcpyAsync(&bits, word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(c, cudaMemcpyAsync(c->result, word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     const cf_status s = wait_stream(c);
     if (s != CF_OK) return s;
     float d2;
-    std::memcpy(&d2, &bits, sizeof d2);
+    std::memcpy(&d2, c->result, sizeof d2);
     out[0] = std::sqrt((double)d2);
     out[1] = (out[0] - d_ref) / d_ref;
     return CF_OK;

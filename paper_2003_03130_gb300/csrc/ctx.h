@@ -106,9 +106,10 @@ struct cf_ctx {
     size_t mat_cap = 0;              // entries allocated in mat
     float4 *mat = nullptr;
     int *csr_ptr = nullptr, *csr_idx = nullptr, *csr_cursor = nullptr;
-    double *energy_partial = nullptr, *energy_out = nullptr;
+    double *energy_partial = nullptr;
     double *stage = nullptr;  // [3 V] doubles for host <-> device vertex arrays
-    double *taylor_partial = nullptr, *taylor_out = nullptr;
+    double *taylor_partial = nullptr;
+    double *result = nullptr;  // [10] mapped page-locked: scalar results, written there by the kernels themselves
 
     // force regions: three slots of region_stride words, each the bitset over
     // the tiles of the current tiling (region_bits_max words for the tiling
