@@ -25,7 +25,7 @@
 // Bound by instruction issue (0.6 of the slots: ~400 instructions a tet, ~40
 // an incidence). 64 cells of 8.3 k tets (1,853 vertices) on 128 SMs: 17.5 us a
 // step, where the three launches took 29 (the corner forces cross L2 there, 64
-// bytes written and read per tet); a reverse step 36 us, 53 before. Two cells
+// bytes written and read per tet); a reverse step 30 us, 53 before. Two cells
 // of 1.2 k tets: 5 to 6 us a step of either kind, 15 and 25 before. Velocities
 // stay in shared memory and the trail is stored a step late, since a barrier's
 // release waits for every store still on its way (19 -> 17.5 us). Measured and
