@@ -91,7 +91,7 @@ KERNELS = ("k_tet_force", "k_gather_spread", "k_lbm_far", "k_lbm_near", "k_inter
 def parse():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
-    ap.add_argument("--steps", type=int, default=20000)
+    ap.add_argument("--steps", type=int, default=2000)
     ap.add_argument("--warmup", type=int, default=200)
     ap.add_argument("--impl", choices=("ours", "reference"), default="ours")
     ap.add_argument("--n", type=int, default=128, help="cubic lattice extent")
@@ -845,9 +845,9 @@ def compression_measure(fit_iters):
         "forward_s": fwd_s,
         "config": {"workload": f"compression_{len(ids)}cells_R10", "n_tets": ntets, "levels": len(cs.strains),
                    "steps_per_level": cs.steps, "max_strain": cs.strains[-1], "parallelism": "replicas",
-                   "l2": "working set ~30 MB, fits L2 (latency-bound relaxation)"},
+                   "l2": "working set ~30 MB, fits L2 (cells on chip, bound by instruction issue)"},
         "tet_forces_per_s": ntets * nsteps / fwd_s,
-        "gpu_launches": 3 * nsteps,
+        "gpu_launches": len(cs.strains) * (cs.ramp + 1),  # one per plate move: a move's steps run in one launch
         "adjoint": {
             "backward_s": float(np.median(bwd)) if bwd else None,
             "forward_s": fwd_s,
