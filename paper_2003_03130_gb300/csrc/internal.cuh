@@ -501,7 +501,7 @@ cudaError_t launch_relax_cells(const RelaxPlan &pl, const MeshView &m, const flo
                                float c, float kp, const float *zlo, const float *zhi, unsigned *err, cudaStream_t s);
 cudaError_t launch_relax_reverse(const RelaxPlan &pl, const MeshView &m, const float4 *y, float4 *ly, float4 *lv, int n,
                                  float dt, float c, float kp, const float *zlo, const float *zhi, double *grad,
-                                 cudaStream_t s);
+                                 unsigned *err, cudaStream_t s);
 
 cudaError_t launch_lbm_init(void *f, const LbmParams &p, cudaStream_t s);
 // rho and u(t) of every node after a step. u is u(t) as the near field

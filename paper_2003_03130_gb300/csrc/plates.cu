@@ -383,7 +383,7 @@ cf_status cf_relax_adjoint(cf_ctx *c, const double *dF) {
                                                c->seg, nullptr, len - 1, e.dt, e.c, e.kp, c->zlo, c->zhi, c->d_err,
                                                c->stream));
             CUDA_TRY(c, launch_relax_reverse(*pl, m, c->seg, c->lam, c->lamv, len, e.dt, e.c, e.kp, c->zlo, c->zhi,
-                                             c->grad, c->stream));
+                                             c->grad, c->d_err, c->stream));
             continue;
         }
         CUDA_TRY(c, cudaMemcpyAsync(c->segv, ck + V, sizeof(float4) * V, cudaMemcpyDeviceToDevice, c->stream));

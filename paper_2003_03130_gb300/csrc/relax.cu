@@ -312,7 +312,8 @@ __global__ void __launch_bounds__(kStepBlock, 1)
 // gradients += dt m . df/d(mu, kappa, w).
 __global__ void __launch_bounds__(kReverseBlock, 1)
     k_relax_reverse(RelaxPlan pl, MeshView m, const float4 *__restrict__ y, float4 *ly, float4 *lv, int n, float dt,
-                    float c, float kp, const float *__restrict__ zlo, const float *__restrict__ zhi, double *grad) {
+                    float c, float kp, const float *__restrict__ zlo, const float *__restrict__ zhi, double *grad,
+                    unsigned *err) {
     extern __shared__ float4 su[];  // [vertices of the cell] displacements, then m, then the corner tangents
     __shared__ Sum2 part[3][kReverseBlock / 32];
     const cg::cluster_group cluster = cg::this_cluster();
@@ -373,7 +374,10 @@ __global__ void __launch_bounds__(kReverseBlock, 1)
             __syncwarp();                         // the four lanes have read ly
             if (!live) continue;
             for (int r = lane; r < pl.cs; r += 4) *cluster.map_shared_rank(sm + local, r) = mn;
-            if (lane == 0) ly[v] = a;
+            if (lane == 0) {
+                ly[v] = a;
+                if (!isfinite(jx + jy + jz)) atomicOr(err, ERR_NONFINITE);  // as the general path's vertex sums
+            }
             if (lane == 1) lv[v] = b;
         }
         cluster.sync();
@@ -428,10 +432,10 @@ cudaError_t launch_relax_cells(const RelaxPlan &pl, const MeshView &m, const flo
 
 cudaError_t launch_relax_reverse(const RelaxPlan &pl, const MeshView &m, const float4 *y, float4 *ly, float4 *lv, int n,
                                  float dt, float c, float kp, const float *zlo, const float *zhi, double *grad,
-                                 cudaStream_t s) {
+                                 unsigned *err, cudaStream_t s) {
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = relax_config(pl, kReverseBlock, pl.smem_reverse, &attr, s);
-    return cudaLaunchKernelEx(&cfg, k_relax_reverse, pl, m, y, ly, lv, n, dt, c, kp, zlo, zhi, grad);
+    return cudaLaunchKernelEx(&cfg, k_relax_reverse, pl, m, y, ly, lv, n, dt, c, kp, zlo, zhi, grad, err);
 }
 
 // True if a cluster of the plan can be resident (its blocks must be at once).
