@@ -814,6 +814,9 @@ def compression_measure(fit_iters):
     run = Compression(ctx, ids, y0, z_lo, radius, cs.strains, cs.steps, cs.dt, cs.k_plate, cs.ramp, cs.damping)
     nsteps = len(cs.strains) * cs.steps
     target = run.run(cs.hidden_mu, cs.hidden_kappa, cs.hidden_w, record=False)  # warm-up and target curves
+    path = P.cf_get_relax_path(ctx)
+    moves = [n for _, n, _ in configs.plate_schedule(z_lo, radius, cs.strains, cs.steps, cs.ramp) if n]
+    launches = sum(-(-n // path["steps_per_launch"]) if path["step_blocks"] else 3 * n for n in moves)
     clocks = ClockSampler(0)
     clocks.start()
     t0 = time.perf_counter()
@@ -847,7 +850,7 @@ def compression_measure(fit_iters):
                    "steps_per_level": cs.steps, "max_strain": cs.strains[-1], "parallelism": "replicas",
                    "l2": "working set ~30 MB, fits L2 (cells on chip, bound by instruction issue)"},
         "tet_forces_per_s": ntets * nsteps / fwd_s,
-        "gpu_launches": len(cs.strains) * (cs.ramp + 1),  # one per plate move: a move's steps run in one launch
+        "gpu_launches": launches,  # of the relaxation steps
         "adjoint": {
             "backward_s": float(np.median(bwd)) if bwd else None,
             "forward_s": fwd_s,

@@ -397,6 +397,15 @@ cf_status cf_plates_set(cf_ctx *ctx, double k_plate, const double *z_lo, const d
  * stiffness), CF_EINVERTED if a tet inverts. */
 cf_status cf_relax(cf_ctx *ctx, int32_t n, double dt, double damping, int32_t record);
 
+/* How the relaxation steps of the current cells run, path[CF_RELAX_PATH_LEN]:
+ * path[0], path[1]: thread blocks per cell with which steps and reverse steps
+ * keep a cell's state on chip, 0 where they take launches of their own for
+ * every step (three for a step); path[2]: steps of one launch on chip, at most
+ * (a recorded call: one launch per checkpoint). The results of a step are the
+ * same bits either way. CF_ESTATE without cells. */
+#define CF_RELAX_PATH_LEN 3
+cf_status cf_get_relax_path(cf_ctx *ctx, int32_t *path);
+
 /* Top-plate force per cell at the current positions, out[ncells]. */
 cf_status cf_plate_force(cf_ctx *ctx, double *out);
 

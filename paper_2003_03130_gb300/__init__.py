@@ -81,6 +81,7 @@ def lib():
             "cf_last_error": ([vp], ctypes.c_char_p),
             "cf_plates_set": ([vp, ctypes.c_double, _d, _d], ctypes.c_int),
             "cf_relax": ([vp, ctypes.c_int32, ctypes.c_double, ctypes.c_double, ctypes.c_int32], ctypes.c_int),
+            "cf_get_relax_path": ([vp, ctypes.POINTER(ctypes.c_int32)], ctypes.c_int),
             "cf_plate_force": ([vp, _d], ctypes.c_int),
             "cf_tape_clear": ([vp], ctypes.c_int),
             "cf_tape_generation": ([vp, ctypes.POINTER(ctypes.c_int64)], ctypes.c_int),
@@ -456,6 +457,14 @@ def cf_plates_set(ctx, k_plate, z_lo, z_hi):
 
 def cf_relax(ctx, n, dt, damping=0.0, record=False):
     _check(ctx, lib().cf_relax(ctx.handle, n, dt, damping, 1 if record else 0))
+
+
+def cf_get_relax_path(ctx):
+    """Blocks per cell of on-chip relaxation steps and reverse steps (0: launches of their own for every step), and
+    steps of one launch on chip."""
+    path = (ctypes.c_int32 * 3)()
+    _check(ctx, lib().cf_get_relax_path(ctx.handle, path))
+    return {"step_blocks": path[0], "reverse_blocks": path[1], "steps_per_launch": path[2]}
 
 
 def cf_plate_force(ctx):

@@ -322,6 +322,19 @@ cf_status cf_relax(cf_ctx *c, int32_t n, double dt, double damping, int32_t reco
     return consume_errors(c);
 }
 
+cf_status cf_get_relax_path(cf_ctx *c, int32_t *path) {
+    cf_status st = need_cells(c);
+    if (st != CF_OK) return st;
+    DeviceGuard dg(c->device);
+    if (!path) return fail(c, CF_EINVAL, "null output");
+    st = make_plan(c);
+    if (st != CF_OK) return st;
+    const RelaxPlan *pl = plan_of(c);
+    path[0] = path[1] = pl ? pl->cs : 0;
+    path[2] = kRelaxSteps;
+    return CF_OK;
+}
+
 cf_status cf_plate_force(cf_ctx *c, double *out) {
     cf_status st = need_cells(c);
     if (st != CF_OK) return st;
