@@ -482,6 +482,7 @@ struct RelaxPart {
 };
 struct RelaxPlan {
     int cs, nparts, NT;      // blocks per cell, parts, tets of all parts
+    bool steps, reverse;     // steps, reverse steps are taken on chip
     int per_tet;             // tets have material slots of their own (MeshView::tmat)
     size_t smem_step, smem_reverse;
     const RelaxPart *parts;  // [nparts], cs per cell
@@ -491,7 +492,7 @@ struct RelaxPlan {
 };
 size_t relax_smem(int cell_nv, int nv, int nt, bool reverse);
 cudaError_t prepare_relax(int smem_max);
-bool relax_fits(const RelaxPlan &pl);
+int relax_clusters(const RelaxPlan &pl);
 cudaError_t launch_relax_count(const MeshView &m, const int4 *cells, int ncells, int *counts, int *degree,
                                cudaStream_t s);
 cudaError_t launch_relax_fill(const MeshView &m, const RelaxPart *parts, int nparts, int cs, const int4 *cells,

@@ -12,13 +12,15 @@
 //   lambda_y <- lambda_y + dt (J_el + J_plate) m, lambda_v <- c m,
 // accumulating dt m . df/d(mu, kappa, w) per cell in double.
 #include <algorithm>
+#include <functional>
+#include <queue>
 
 #include "ctx.h"
 
 namespace {
 
 constexpr int kTapeStride = 50;
-constexpr int kRelaxSteps = 1000;  // steps of one launch, at most (some 10 ms)
+constexpr int kRelaxSteps = 1000;  // steps of one launch, at most (3 to 20 ms a wave of cells)
 
 void free_adjoint(cf_ctx *c) {
     for (auto *p : c->ckpt) cudaFree(p);
@@ -87,11 +89,50 @@ cf_status ensure_adjoint(cf_ctx *c) {
     return CF_OK;
 }
 
-// The on-chip relaxation's plan for the current mesh, if it fits: cells cut
-// into `cs` blocks, the fewest that hold a part in shared memory; more, up to
-// eight, while every block still gets an SM of its own and a part has more
-// tets than threads. A mesh that does not fit, or no memory for the plan,
-// leaves the general path.
+// Time of a step on chip and of a step in launches of their own, microseconds:
+// a + tet t + vertex v, for the tets of a cell's largest block (a cluster's
+// step) or for all tets and vertices (the launches of a step, bound by their
+// latency up to some 50 k tets: `least`). Fitted to 110 sets of cells on GB300
+// (1 to 2,000 cells of 192 to 13.6 k tets, equal ones and one large cell among
+// small ones), which they meet within 19 %; a reverse step includes the
+// recomputed forward one.
+struct StepTime {
+    double least, a, tet, vertex;
+};
+constexpr StepTime kChipStep{0.0, 2.15, 2.92e-3, 0.0}, kChipReverse{0.0, 4.9, 8.6e-3, 0.0};
+constexpr StepTime kLaunchStep{12.4, 10.9, 3.4e-5, 1.8e-5}, kLaunchReverse{25.0, 25.8, 5.9e-5, 1.47e-4};
+
+double step_time(const StepTime &q, double nt, double nv) {
+    return std::max(q.least, q.a + q.tet * nt + q.vertex * nv);
+}
+
+// Time of a step on chip of cells whose largest blocks hold nt tets, `slots`
+// clusters at a time, the next cell on the slot that is free first.
+double on_chip_time(const StepTime &q, const std::vector<int> &nt, int slots) {
+    std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
+    double end = 0.0;
+    for (const int n : nt) {
+        double t = step_time(q, n, 0);
+        if ((int)busy.size() == slots) {
+            t += busy.top();
+            busy.pop();
+        }
+        busy.push(t);
+        end = std::max(end, t);
+    }
+    return end;
+}
+
+// The on-chip relaxation's plan for the current mesh, if it fits and is
+// expected to be faster: cells cut into `cs` blocks, the fewest that hold a
+// part in shared memory; more, up to eight, while every block still gets an SM
+// of its own and a part has more than kRelaxRound tets. The cells of a mesh
+// share cs, and a block has its SM to itself, so many small cells run in
+// waves, and one large cell cuts the small ones beside it too. Steps and
+// reverse steps go on chip each where the estimates above say so. Measured,
+// on chip against three launches a step: 64 cells of 8.3 k tets 16.3 and 28.9
+// us, reverse steps 47 and 70; 2,000 cells of 192 tets 36.9 and 25.8, reverse
+// 88 and 66; 300 of 192 beside one of 13.6 k 50 and 14.5, reverse 121 and 35.
 cf_status make_plan(cf_ctx *c) {
     if (c->plan_state) return CF_OK;
     c->plan_state = 2;
@@ -140,16 +181,15 @@ cf_status make_plan(cf_ctx *c) {
     TRY_P(cudaMemcpyAsync(counts.data(), d_counts, sizeof(int) * counts.size(), cudaMemcpyDeviceToHost, c->stream));
     TRY_P(cudaStreamSynchronize(c->stream));
     if (counts.back() > kRelaxDegree) return done(cudaSuccess);
+    std::vector<int> most_of(C);  // tets of a cell's largest block
     auto largest = [&](int cs, bool &fits) {
-        int most = 0;
         fits = true;
-        for (int k = 0; k < C; ++k)
-            for (int r = 0; r < cs; ++r) {
-                const int nt = counts[15 * (size_t)k + cs - 1 + r];
-                most = std::max(most, nt);
-                if (relax_smem(cells[k].y, cells[k].y, nt, true) > (size_t)(smem - kRelaxStatic)) fits = false;
-            }
-        return most;
+        for (int k = 0; k < C; ++k) {
+            const int *n = counts.data() + 15 * (size_t)k + cs - 1;
+            most_of[k] = *std::max_element(n, n + cs);
+            if (relax_smem(cells[k].y, cells[k].y, most_of[k], true) > (size_t)(smem - kRelaxStatic)) fits = false;
+        }
+        return *std::max_element(most_of.begin(), most_of.end());
     };
     int cs = 1;
     bool fits = false;
@@ -177,7 +217,12 @@ cf_status make_plan(cf_ctx *c) {
         }
     if (nt_all > INT_MAX) return done(cudaSuccess);
     pl.NT = (int)nt_all;
-    if (!relax_fits(pl)) return done(cudaSuccess);
+    const int slots = relax_clusters(pl);
+    if (slots == 0) return done(cudaSuccess);
+    largest(cs, fits);
+    pl.steps = on_chip_time(kChipStep, most_of, slots) < step_time(kLaunchStep, c->T, c->V);
+    pl.reverse = on_chip_time(kChipReverse, most_of, slots) < step_time(kLaunchReverse, c->T, c->V);
+    if (!pl.steps && !pl.reverse) return done(cudaSuccess);
     TRY_P(dalloc(&c->plan_parts, parts.size()));
     TRY_P(dalloc(&c->plan_rows, 3 * (size_t)pl.NT));
     TRY_P(dalloc(&c->plan_list, pl.NT));
@@ -198,9 +243,10 @@ cf_status make_plan(cf_ctx *c) {
     return done(cudaSuccess);
 }
 
-// The plan if the mesh has one, with the materials' present form.
-const RelaxPlan *plan_of(cf_ctx *c) {
-    if (c->plan_state != 1) return nullptr;
+// The plan if the mesh has one that takes steps (reverse: reverse steps) on
+// chip, with the materials' present form.
+const RelaxPlan *plan_of(cf_ctx *c, bool reverse) {
+    if (c->plan_state != 1 || !(reverse ? c->plan.reverse : c->plan.steps)) return nullptr;
     c->plan.per_tet = 0;
     for (const CellInfo &ci : c->cells) c->plan.per_tet |= ci.per_tet;
     return &c->plan;
@@ -296,7 +342,7 @@ cf_status cf_relax(cf_ctx *c, int32_t n, double dt, double damping, int32_t reco
     }
     st = make_plan(c);
     if (st != CF_OK) return st;
-    const RelaxPlan *pl = plan_of(c);
+    const RelaxPlan *pl = plan_of(c, false);
     for (int k = 0; pl && k < n;) {  // on chip: a launch per checkpoint, or per kRelaxSteps
         const int b = std::min(record ? kTapeStride : kRelaxSteps, n - k);
         CUDA_TRY(c, launch_relax_cells(*pl, m, u, c->vel_r, u, c->vel_r,
@@ -329,8 +375,8 @@ cf_status cf_get_relax_path(cf_ctx *c, int32_t *path) {
     if (!path) return fail(c, CF_EINVAL, "null output");
     st = make_plan(c);
     if (st != CF_OK) return st;
-    const RelaxPlan *pl = plan_of(c);
-    path[0] = path[1] = pl ? pl->cs : 0;
+    path[0] = plan_of(c, false) ? c->plan.cs : 0;
+    path[1] = plan_of(c, true) ? c->plan.cs : 0;
     path[2] = kRelaxSteps;
     return CF_OK;
 }
@@ -383,7 +429,7 @@ cf_status cf_relax_adjoint(cf_ctx *c, const double *dF) {
     CUDA_TRY(c, launch_adj_seed(m, c->ckpt[e.ck0 + e.nck - 1], e.kp, c->zlo, c->zhi, c->dF, c->lam, c->stream));
     st = make_plan(c);
     if (st != CF_OK) return st;
-    const RelaxPlan *pl = plan_of(c);
+    const RelaxPlan *pl = plan_of(c, true);
     if (!pl) CUDA_TRY(c, launch_adj_m(c->V, c->lam, c->lamv, e.dt, c->mvec, c->stream));
     for (int j = e.nck - 2; j >= 0; --j) {
         const int s0 = j * kTapeStride, len = std::min(kTapeStride, e.n - s0);

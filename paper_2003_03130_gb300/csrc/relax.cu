@@ -18,9 +18,10 @@
 // per vertex, a fixed tree), and the tets run the same code, so the positions
 // are those of the general path (three launches a step, k_tet_force,
 // k_gather_spread, k_plate_step), bit for bit. That path stays for cells
-// that do not fit: shared memory holds 16 bytes per vertex of the cell, 16 more
-// per vertex and 36 per tet of a block (the reverse step 32 and 36), up to eight blocks a
-// cluster, 65,535 vertices a cell and 32 incidences a vertex.
+// that do not fit (shared memory holds 16 bytes per vertex of the cell, 16 more
+// per vertex and 36 per tet of a block, the reverse step 32 and 36; up to eight
+// blocks a cluster, 65,535 vertices a cell and 32 incidences a vertex) and
+// where it is expected to be faster (csrc/plates.cu, make_plan).
 //
 // Bound by instruction issue (0.6 of the slots: ~400 instructions a tet, ~40
 // an incidence). 64 cells of 8.3 k tets (1,853 vertices) on 128 SMs: 17.5 us a
@@ -438,8 +439,9 @@ cudaError_t launch_relax_reverse(const RelaxPlan &pl, const MeshView &m, const f
     return cudaLaunchKernelEx(&cfg, k_relax_reverse, pl, m, y, ly, lv, n, dt, c, kp, zlo, zhi, grad, err);
 }
 
-// True if a cluster of the plan can be resident (its blocks must be at once).
-bool relax_fits(const RelaxPlan &pl) {
+// Clusters of the plan that can be resident at a time (a cluster's blocks must
+// be at once); 0: none.
+int relax_clusters(const RelaxPlan &pl) {
     cudaLaunchAttribute attr;
     int a = 0, b = 0;
     const cudaLaunchConfig_t f = relax_config(pl, kStepBlock, pl.smem_step, &attr, nullptr);
@@ -447,7 +449,7 @@ bool relax_fits(const RelaxPlan &pl) {
     const cudaLaunchConfig_t r = relax_config(pl, kReverseBlock, pl.smem_reverse, &attr, nullptr);
     if (cudaOccupancyMaxActiveClusters(&b, k_relax_reverse, &r) != cudaSuccess) b = 0;
     cudaGetLastError();
-    return a > 0 && b > 0;
+    return a < b ? a : b;
 }
 
 }  // namespace cf
