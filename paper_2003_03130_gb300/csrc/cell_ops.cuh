@@ -29,7 +29,8 @@ __device__ __forceinline__ void tet_load(const MeshView &m, const float4 *__rest
 }
 
 // Corner forces of tet t from its inputs (Sec. 3.1): f^a = -V0 P B_a,
-// f^4 = -(f^1 + f^2 + f^3).
+// f^4 = -(f^1 + f^2 + f^3). KEEP: see mr_cofactor.
+template <bool KEEP = false>
 __device__ __forceinline__ void tet_corners(const MeshView &m, const TetIn &in, unsigned *err, int t, float (&f)[4][3]) {
     float H[3][3];
     tet_grad(in.w[0], in.w[1], in.w[2], in.w[3], in.Bm, H);
@@ -38,23 +39,25 @@ __device__ __forceinline__ void tet_corners(const MeshView &m, const TetIn &in, 
     invariants_t(H, v);
     if (needs_fp64_volume(m, in.mat))
         set_volume_change(v, (float)volume_change64(m.B64, m.T, t, in.w[0], in.w[1], in.w[2], in.w[3]));
-    mr_stress_inv(H, in.mat.x, in.mat.y, in.mat.z, v, P);
+    mr_stress_inv<KEEP>(H, in.mat.x, in.mat.y, in.mat.z, v, P);
     if (!(v.J > 0.f)) atomicOr(err, ERR_INVERTED);
     corner_forces(P, in.Bm, in.V0, f);
 }
 
+template <bool KEEP = false>
 __device__ __forceinline__ void tet_forces_store(const MeshView &m, const TetIn &in, unsigned *err, int t) {
     float f[4][3];
-    tet_corners(m, in, err, t, f);
+    tet_corners<KEEP>(m, in, err, t, f);
 #pragma unroll
     for (int a = 0; a < 4; ++a) m.fc[a * m.T + t] = make_float4(f[a][0], f[a][1], f[a][2], 0.f);
 }
 
+template <bool KEEP = false>
 __device__ __forceinline__ void tet_corner_forces(const MeshView &m, const float4 *__restrict__ u, unsigned *err,
                                                   int t) {
     TetIn in;
     tet_load(m, u, t, in);
-    tet_forces_store(m, in, err, t);
+    tet_forces_store<KEEP>(m, in, err, t);
 }
 
 // The per-vertex part of K1 when it marks the region: add the next step's

@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kChainBlock, 4)
                 if (mark.bits)
                     for (int v = x.z + threadIdx.x; v < x.w; v += kChainBlock) mark_vertex<W>(m, u, lp, v, mark);
             } else if (x.x == 1) {
-                for (int t = x.z + threadIdx.x; t < x.w; t += kChainBlock) tet_corner_forces(m, u, err, t);
+                for (int t = x.z + threadIdx.x; t < x.w; t += kChainBlock) tet_corner_forces<true>(m, u, err, t);
             } else {
                 for (int v0 = x.z; v0 < x.w; v0 += kChainBlock / 4) {  // the whole block takes each round
                     const int v = v0 + (threadIdx.x >> 2);

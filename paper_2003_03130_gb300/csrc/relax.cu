@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kStepBlock, 1)
             if (by_index) t = __ldg(pl.list + p.t0 + i) & INT_MAX;
             in.mat = pl.per_tet ? __ldg(m.mat + __ldg(m.tmat + t)) : cell_mat;
             float f[4][3];
-            tet_corners(m, in, err, t, f);
+            tet_corners<true>(m, in, err, t, f);
 #pragma unroll
             for (int k = 0; k < 9; ++k) fc[9 * i + k] = f[k / 3][k % 3];
         }
