@@ -164,11 +164,19 @@ void shape_to_lbm(LbmParams &p, const Shape &sh) {
     p.pairs = sh.pop_pairs;
 }
 
-// The lattice of a step of parity p: the direction of its sweep, and (alone:
-// a run without cells, whose data nothing else in L2 competes with) always to
-// and fro.
-LbmParams sweep(LbmParams q, int p, bool alone = false) {
-    q.turn |= alone;
+// The lattice of a step of parity p: whether it is swept to and fro, and the
+// step's direction. With cells from both buffers larger than L2 (turn); a run
+// of the fluid alone (alone), whose data nothing else in L2 competes with,
+// from half of that, but not node pairs in rows that leave a third of a block
+// or more idle: issue bounds them there (csrc/lbm.cu has the figures).
+LbmParams sweep(const cf_ctx *c, int p, bool alone = false) {
+    LbmParams q = c->lp;
+    if (alone) {
+        const int pairs = q.nx / 2, block = std::min(pairs, 64);
+        const bool idle = pop_bytes(q.fmt) == 2 && q.pairs && q.nx % 2 == 0 &&
+                          3 * pairs < 2 * block * ((pairs + block - 1) / block);
+        q.turn = 2 * pop_bytes(q.fmt) * 19 * (size_t)q.N > (size_t)c->l2_bytes / 2 && !idle;
+    }
     q.back = q.turn && p;
     return q;
 }
@@ -196,7 +204,7 @@ cf_status enqueue_steps(cf_ctx *c, Kind kind, int p0, int s0, int nsteps, cudaSt
     if (kind == Kind::Fluid) {
         for (int i = 0; i < nsteps; ++i) {
             const int p = p0 ^ (i & 1);
-            CUDA_TRY(c, launch_lbm(c->f[p], c->f[1 - p], sweep(c->lp, p, true), c->seed + p, c->seed + 1 - p, sf));
+            CUDA_TRY(c, launch_lbm(c->f[p], c->f[1 - p], sweep(c, p, true), c->seed + p, c->seed + 1 - p, sf));
         }
         return CF_OK;
     }
@@ -215,7 +223,7 @@ cf_status enqueue_steps(cf_ctx *c, Kind kind, int p0, int s0, int nsteps, cudaSt
         const int p = p0 ^ (i & 1), s = (s0 + i) % 3;
         const RegionSlot use = region_slot(c, s), acc = accum_slot(c, s);
         if (i > 0) CUDA_TRY(c, cudaStreamWaitEvent(sf, ev_near[i - 1], 0));
-        CUDA_TRY(c, launch_lbm_far(c->f[p], c->f[1 - p], sweep(c->lp, p), use.bits, c->seed + p, sh.far_spec, sf));
+        CUDA_TRY(c, launch_lbm_far(c->f[p], c->f[1 - p], sweep(c, p), use.bits, c->seed + p, sh.far_spec, sf));
         CUDA_TRY(c, cudaEventRecord(ev_far[i], sf));
         if (!(first && i == 0)) {  // K5 of the previous step (parity 1-p), with mark_k5 marking acc
             CUDA_TRY(c, launch_interp_advect(m, c->vel, c->lp, c->u[1 - p], c->u[p], c->d_err, sc, sh.interp_block,
@@ -224,7 +232,7 @@ cf_status enqueue_steps(cf_ctx *c, Kind kind, int p0, int s0, int nsteps, cudaSt
         if (first && i == 0 && !sh.mark_k5) CUDA_TRY(c, clear_slot(c, acc, sc));
         CUDA_TRY(c, launch_chain_step(c, m, p, sh, acc, sc));
         if (i > 0) CUDA_TRY(c, cudaStreamWaitEvent(sc, ev_far[i - 1], 0));
-        CUDA_TRY(c, launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c->lp, p), use.bits, c->vel,
+        CUDA_TRY(c, launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c, p), use.bits, c->vel,
                                     sh.near_rows || !c->near_tiles_fit ? 0 : near_grid(c), c->seed + p, c->seed + 1 - p, next_slot(c, s).bits, sc));
         CUDA_TRY(c, cudaEventRecord(ev_near[i], sc));
     }
@@ -499,9 +507,8 @@ cf_status cf_lbm_init(cf_ctx *c, int32_t nx, int32_t ny, int32_t nz, double tau,
         tmax = std::max(tmax, tiles_of(p));
     }
     shape_to_lbm(p, c->shape);
-    int l2 = 0;
-    cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device);
-    p.turn = 2 * 19 * (long long)pop_bytes(p.fmt) * N > (long long)l2;  // both buffers
+    cudaDeviceGetAttribute(&c->l2_bytes, cudaDevAttrL2CacheSize, c->device);
+    p.turn = 2 * 19 * (long long)pop_bytes(p.fmt) * N > (long long)c->l2_bytes;  // both buffers
     c->region_bits_max = (tmax + 31) / 32;
     c->region_stride = (c->region_bits_max + 31) / 32 * 32;
     int smem_optin = 0;
@@ -983,11 +990,11 @@ cf_status timed_steps(cf_ctx *c, int n, const Shape &sh, double acc[5]) {
                 e = launch_gather_spread(m, c->u[p], c->F, &c->lp, c->d_err, s, sh.gather_block, sh.staged);
             cudaEventRecord(E[3], s);
             if (e == cudaSuccess)
-                e = cells ? launch_lbm_far(c->f[p], c->f[1 - p], sweep(c->lp, p), use.bits, c->seed + p, sh.far_spec, s)
-                          : launch_lbm(c->f[p], c->f[1 - p], sweep(c->lp, p, true), c->seed + p, c->seed + 1 - p, s);
+                e = cells ? launch_lbm_far(c->f[p], c->f[1 - p], sweep(c, p), use.bits, c->seed + p, sh.far_spec, s)
+                          : launch_lbm(c->f[p], c->f[1 - p], sweep(c, p, true), c->seed + p, c->seed + 1 - p, s);
             cudaEventRecord(E[4], s);
             if (cells && e == cudaSuccess)
-                e = launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c->lp, p), use.bits, c->vel,
+                e = launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c, p), use.bits, c->vel,
                                     sh.near_rows || !c->near_tiles_fit ? 0 : near_grid(c), c->seed + p, c->seed + 1 - p,
                                     next_slot(c, sph).bits, s);
             cudaEventRecord(E[5], s);

@@ -122,6 +122,7 @@ struct cf_ctx {
     bool near_tiles_fit = true;
     Shape shape;
     int sms = 152;  // multiprocessors of the device
+    int l2_bytes = 0;
 
     // compression between plates and its adjoint (csrc/plates.cu)
     struct TapeEntry {

@@ -80,7 +80,7 @@ struct LbmParams {
     int l2;             // FP32 far and near fields: populations cached in L2 at normal priority
                         // (1) instead of streamed with evict-first hints (0)
     int pairs;          // 16-bit formats, nx even: two nodes per thread in the row-form kernels
-    int turn, back;     // sweep z to and fro (a lattice larger than L2); this step backwards
+    int turn, back;     // swept along z to and fro, results kept in L2; this step backwards
     int det;            // deterministic spread: the force field in fixed point, long long [3][N]
     // force-region tiles of 2^tlx x 2^tly x 2^tlz = 256 nodes (x fastest;
     // the last tile of an axis may stick out of the lattice), ntx * nty * ntz

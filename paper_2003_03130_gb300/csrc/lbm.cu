@@ -16,10 +16,12 @@
 // equilibrium (FP32 rounding then scales with the O(u) signal), in FP32, or in
 // FP16 / BF16 multiplied by a power of two per weight class (2^14, 2^16, 2^17
 // for w = 1/3, 1/18, 1/36, so that the stored values are O(10^3) and never
-// subnormal in FP16); the collide always runs in FP32. Population loads and
-// stores carry the streaming cache hint (evict first): every population is
-// touched once per step, and the hint keeps the cells' few MB of mesh data
-// resident in L2 while the lattice streams through it.
+// subnormal in FP16); the collide always runs in FP32. Population loads
+// carry the streaming cache hint (evict first), and so do the stores of a
+// lattice that fits L2 beside cells: every population is touched once per
+// step, and the hint keeps the cells' few MB of mesh data resident in L2 while
+// the lattice streams through it. Other lattices are swept to and fro and keep
+// their results (KEEP below).
 //
 // One node per thread: 19 independent coalesced loads per node (x-shifted
 // rows are off by one word; neighbouring warps share the lines in L2), the
@@ -47,33 +49,26 @@ namespace cf {
 // unbiased (exact for FP16-normal values). The caller passes a zero dither
 // for non-finite values, which then convert as they are.
 //
-// Stores carry an L2 policy (p.turn): a lattice larger than L2 is swept along
-// +z and -z in turn (the parity of the step), the sources read evict-first and
-// the results stored at normal priority, so that a sweep starts on the planes
-// that the one before left in L2 (128^3 FP32: the fluid alone 50.4 -> 45.8 us a
-// step, with a cell 56.3 -> 53.2; 256x128x128 FP16 66.3 -> 63.7; 160x240x80 80.7
-// -> 78.2). In a lattice that fits, normal-priority stores only evict the
-// cells' data (80x128x64 with 8 cells 41.8 -> 43.6), so there they stay
-// evict-first.
-typedef unsigned long long Policy;
-
-__device__ __forceinline__ Policy store_policy(const LbmParams &p) {
-    Policy q;
-    if (p.turn)
-        asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(q));
+// KEEP: results stored at normal L2 priority (sources are always read
+// evict-first), for a lattice that is swept along +z and -z in turn
+// (LbmParams::turn, by the parity of the step): a sweep starts on the planes
+// that the one before left in L2. The fluid alone gains from half of L2 for
+// both buffers (FP32 80^3 12.2 -> 11.8 us a step, 96^3 20.4 -> 17.4, 128^3
+// 50.1 -> 45.5, 192^3 163.7 -> 159.8; FP16 104^3 17.2 -> 16.6, 128^3 27.5 ->
+// 25.6), smaller ones nothing, nor node pairs in half-empty blocks (FP16 160^3
+// 71.2 -> 72.0). With cells it is worth it once both buffers exceed L2 (128^3
+// with a cell, FP32 52.4 -> 48.2, FP16 31.4 -> 29.5; FP16 160^3 78.0 -> 77.2);
+// in a lattice that fits, the kept results evict the cells' data (512x64x40
+// FP16 with a cell 21.2 -> 22.0, 80x128x64 FP32 with 8 cells 41.8 -> 43.6).
+// KEEP is a template argument: a policy operand on each store cost a 16-bit
+// step 1 to 2 % and 32^3 FP32 7 %, a branch around the stores the node pairs
+// up to 4 %, and a lattice that is not swept needs none of it.
+template <bool KEEP, class T>
+__device__ __forceinline__ void st_pop(T *p, T v) {
+    if (KEEP)
+        *p = v;
     else
-        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(q));
-    return q;
-}
-
-__device__ __forceinline__ void st_hint(float *p, float v, Policy q) {
-    asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(p), "f"(v), "l"(q) : "memory");
-}
-__device__ __forceinline__ void st_hint(unsigned *p, unsigned v, Policy q) {
-    asm volatile("st.global.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(q) : "memory");
-}
-__device__ __forceinline__ void st_hint(void *p, unsigned short v, Policy q) {
-    asm volatile("st.global.L2::cache_hint.u16 [%0], %1, %2;" ::"l"(p), "h"(v), "l"(q) : "memory");
+        __stcs(p, v);
 }
 
 template <class T>
@@ -90,16 +85,16 @@ struct Pop<float> {
     static __device__ __forceinline__ float ld(const float *p) {
         return CS ? __ldcs(p) : __ldcg(p);
     }
-    template <bool CS = true>
-    static __device__ __forceinline__ void st(float *p, float v, Policy q) {
+    template <bool KEEP, bool CS = true>
+    static __device__ __forceinline__ void st(float *p, float v) {
         if (CS)
-            st_hint(p, v, q);
+            st_pop<KEEP>(p, v);
         else
             __stcg(p, v);
     }
-    template <bool CS = true>
-    static __device__ __forceinline__ void st_sr(float *p, float v, unsigned, Policy q) {
-        st<CS>(p, v, q);
+    template <bool KEEP, bool CS = true>
+    static __device__ __forceinline__ void st_sr(float *p, float v, unsigned) {
+        st<KEEP, CS>(p, v);
     }
 };
 
@@ -108,13 +103,13 @@ struct Pop<__half> {
     static constexpr int kDropped = 13;
     template <bool CS = true>
     static __device__ __forceinline__ float ld(const __half *p) { return __half2float(__ldcs(p)); }
-    template <bool CS = true>
-    static __device__ __forceinline__ void st(__half *p, float v, Policy q) {
-        st_hint(p, __half_as_ushort(__float2half_rn(v)), q);
+    template <bool KEEP, bool CS = true>
+    static __device__ __forceinline__ void st(__half *p, float v) {
+        st_pop<KEEP>(p, __float2half_rn(v));
     }
-    template <bool CS = true>
-    static __device__ __forceinline__ void st_sr(__half *p, float v, unsigned dither, Policy q) {
-        st_hint(p, __half_as_ushort(__float2half_rz(__uint_as_float(__float_as_uint(v) + dither))), q);
+    template <bool KEEP, bool CS = true>
+    static __device__ __forceinline__ void st_sr(__half *p, float v, unsigned dither) {
+        st_pop<KEEP>(p, __float2half_rz(__uint_as_float(__float_as_uint(v) + dither)));
     }
 };
 
@@ -123,13 +118,13 @@ struct Pop<__nv_bfloat16> {
     static constexpr int kDropped = 16;
     template <bool CS = true>
     static __device__ __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(__ldcs(p)); }
-    template <bool CS = true>
-    static __device__ __forceinline__ void st(__nv_bfloat16 *p, float v, Policy q) {
-        st_hint(p, __bfloat16_as_ushort(__float2bfloat16_rn(v)), q);
+    template <bool KEEP, bool CS = true>
+    static __device__ __forceinline__ void st(__nv_bfloat16 *p, float v) {
+        st_pop<KEEP>(p, __float2bfloat16_rn(v));
     }
-    template <bool CS = true>
-    static __device__ __forceinline__ void st_sr(__nv_bfloat16 *p, float v, unsigned dither, Policy q) {
-        st_hint(p, __bfloat16_as_ushort(__float2bfloat16_rz(__uint_as_float(__float_as_uint(v) + dither))), q);
+    template <bool KEEP, bool CS = true>
+    static __device__ __forceinline__ void st_sr(__nv_bfloat16 *p, float v, unsigned dither) {
+        st_pop<KEEP>(p, __float2bfloat16_rz(__uint_as_float(__float_as_uint(v) + dither)));
     }
 };
 
@@ -274,7 +269,7 @@ __device__ __forceinline__ bool wall_pull(int y, int ny) {
 // ---------------------------------------------------------------- one node
 // store = false: load and collide but write nothing (a node found, after its
 // loads were issued, to belong to the other part of the split).
-template <class T, bool WALL, bool HAS_F, bool CS = true>
+template <class T, bool WALL, bool HAS_F, bool KEEP, bool CS = true>
 __device__ __forceinline__ void lbm_node(const T *__restrict__ fin, T *__restrict__ fout,
                                          float4 *__restrict__ F, const LbmParams &p, int x, int y, int z,
                                          float4 *__restrict__ vel, unsigned seed, bool store = true) {
@@ -308,7 +303,6 @@ __device__ __forceinline__ void lbm_node(const T *__restrict__ fin, T *__restric
     }
     const float3 u = collide<T>(d, Fx, Fy, Fz, p);
     if (!store) return;
-    const Policy pol = store_policy(p);
     if (HAS_F && spread) force_clear(F, p, n);  // consumed: the next step spreads onto zeros
     if (vel) {  // u(t) of this step, for the interpolation at the vertices
         vel[n] = make_float4(u.x, u.y, u.z, 0.f);
@@ -321,13 +315,13 @@ __device__ __forceinline__ void lbm_node(const T *__restrict__ fin, T *__restric
 #pragma unroll
             for (int q = 0; q < 19; ++q) {
                 const unsigned r = (h + (unsigned)q * 0x9e3779b9u) >> (32 - Pop<T>::kDropped);
-                Pop<T>::template st_sr<CS>(fout + q * N + n, d[q], r & mask, pol);
+                Pop<T>::template st_sr<KEEP, CS>(fout + q * N + n, d[q], r & mask);
             }
             return;
         }
     }
 #pragma unroll
-    for (int q = 0; q < 19; ++q) Pop<T>::template st<CS>(fout + q * N + n, d[q], pol);
+    for (int q = 0; q < 19; ++q) Pop<T>::template st<KEEP, CS>(fout + q * N + n, d[q]);
 }
 
 // ---------------------------------------------------------------- node pairs
@@ -445,7 +439,10 @@ __device__ __forceinline__ void collide2(float2 (&d)[19], float2 Fx, float2 Fy, 
 // the even node), their FP32 values, and the rounded or stochastically
 // rounded conversion back.
 __device__ __forceinline__ unsigned ld_pair(const void *p) { return __ldcs(static_cast<const unsigned *>(p)); }
-__device__ __forceinline__ void st_pair(void *p, unsigned v, Policy q) { st_hint(static_cast<unsigned *>(p), v, q); }
+template <bool KEEP>
+__device__ __forceinline__ void st_pair(void *p, unsigned v) {
+    st_pop<KEEP>(static_cast<unsigned *>(p), v);
+}
 
 template <class T>
 __device__ __forceinline__ float2 unpack2(unsigned w);
@@ -493,7 +490,7 @@ __device__ __forceinline__ unsigned pack2_sr(float2 v, unsigned r) {
 }
 
 // Nodes (x0, x0 + 1) of row (y, z): pull, collide, store, as lbm_node.
-template <class T, bool WALL, bool HAS_F>
+template <class T, bool WALL, bool HAS_F, bool KEEP>
 __device__ __forceinline__ void lbm_pair(const T *__restrict__ fin, T *__restrict__ fout, float4 *__restrict__ F,
                                          const LbmParams &p, int x0, int y, int z, float4 *__restrict__ vel,
                                          unsigned seed) {
@@ -542,50 +539,54 @@ __device__ __forceinline__ void lbm_pair(const T *__restrict__ fin, T *__restric
         vel[n0] = make_float4(ux.x, uy.x, uz.x, 0.f);
         vel[n0 + 1] = make_float4(ux.y, uy.y, uz.y, 0.f);
     }
-    const Policy pol = store_policy(p);
     if (p.sr) {
         // random bits per pair and population: the Weyl step h + q 0x9e3779b9
         // of a per-pair hash of the node and the step's seed
         const unsigned h = mix32((unsigned)n0 ^ mix32(seed));
 #pragma unroll
-        for (int q = 0; q < 19; ++q) st_pair(fout + q * N + n0, pack2_sr<T>(d[q], h + (unsigned)q * 0x9e3779b9u), pol);
+        for (int q = 0; q < 19; ++q) st_pair<KEEP>(fout + q * N + n0, pack2_sr<T>(d[q], h + (unsigned)q * 0x9e3779b9u));
         return;
     }
 #pragma unroll
-    for (int q = 0; q < 19; ++q) st_pair(fout + q * N + n0, pack2_rn<T>(d[q]), pol);
+    for (int q = 0; q < 19; ++q) st_pair<KEEP>(fout + q * N + n0, pack2_rn<T>(d[q]));
 }
 
 // ---------------------------------------------------------------- kernels
 // The z plane of a row-form kernel's block row: backwards in every other step
-// of a lattice that is swept to and fro.
-__device__ __forceinline__ int plane_of(const LbmParams &p, int z) { return p.back ? p.nz - 1 - z : z; }
+// of a lattice that is swept to and fro (TURN: it may be).
+template <bool TURN>
+__device__ __forceinline__ int plane_of(const LbmParams &p, int z) {
+    return TURN && p.back ? p.nz - 1 - z : z;
+}
 
 // The near field also empties the region slot of the step after next's
 // marking (nobody reads it any more: it was the region of the step before),
-// so that no memset stands in the chain of a step's kernels. Thread `i` of
-// `n` threads takes its share.
-__device__ __forceinline__ void clear_words(unsigned *w, int nwords, long long i, long long n) {
-    for (; i < nwords; i += n) w[i] = 0u;
+// so that no memset stands in the chain of a step's kernels. The list form
+// does it last, in 32-bit indices: at the start, the 16-bit kernels spilled
+// three times as much.
+__device__ __forceinline__ void clear_words_list(unsigned *w, int nwords) {
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (unsigned)nwords; i += gridDim.x * blockDim.x) w[i] = 0u;
 }
 
-__device__ __forceinline__ void clear_words_rows(unsigned *w, int nwords) {
+__device__ __forceinline__ void clear_words_rows(unsigned *w, int nwords) {  // more threads than words
     const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-    clear_words(w, nwords, b * blockDim.x + threadIdx.x, (long long)gridDim.x * gridDim.y * gridDim.z * blockDim.x);
+    const long long i = b * blockDim.x + threadIdx.x;
+    if (i < nwords) w[i] = 0u;
 }
 
 // Whole lattice, no force field (fluid-only runs).
-template <class T>
+template <class T, bool KEEP>
 __global__ void __launch_bounds__(128) k_lbm(const T *__restrict__ fin, T *__restrict__ fout, LbmParams p,
                                              const unsigned *__restrict__ seed_in, unsigned *__restrict__ seed_out) {
     const unsigned seed = *seed_in;
     if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *seed_out = seed + 1u;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.nx) return;
-    const int y = blockIdx.y, z = plane_of(p, blockIdx.z);
+    const int y = blockIdx.y, z = plane_of<KEEP>(p, blockIdx.z);
     if (y > 0 && y < p.ny - 1)
-        lbm_node<T, false, false>(fin, fout, nullptr, p, x, y, z, nullptr, seed);
+        lbm_node<T, false, false, KEEP>(fin, fout, nullptr, p, x, y, z, nullptr, seed);
     else
-        lbm_node<T, true, false>(fin, fout, nullptr, p, x, y, z, nullptr, seed);
+        lbm_node<T, true, false, KEEP>(fin, fout, nullptr, p, x, y, z, nullptr, seed);
 }
 
 // Node of thread i in tile (tx, ty, tz): x fastest within the tile. False if
@@ -607,27 +608,27 @@ constexpr int kTileBlock = kTileNodes / 2;
 // SPEC: the region test resolves while the populations load (a region
 // node's loads are wasted, a far node saves a round trip before its loads);
 // otherwise a region node returns before loading.
-template <class T, bool SPEC, bool CS = true>
+template <class T, bool SPEC, bool KEEP, bool CS = true>
 __global__ void __launch_bounds__(128) k_lbm_far(const T *__restrict__ fin, T *__restrict__ fout, LbmParams p,
                                                  const unsigned *__restrict__ bits,
                                                  const unsigned *__restrict__ seed_in) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.nx) return;
-    const int y = blockIdx.y, z = plane_of(p, blockIdx.z);
+    const int y = blockIdx.y, z = plane_of<KEEP || !CS>(p, blockIdx.z);
     const bool region = region_has(bits, tile_index(p, x >> p.tlx, y >> p.tly, z >> p.tlz));
     if (!SPEC && region) return;
     const unsigned seed = *seed_in;
     if (y > 0 && y < p.ny - 1)
-        lbm_node<T, false, false, CS>(fin, fout, nullptr, p, x, y, z, nullptr, seed, !region);
+        lbm_node<T, false, false, KEEP, CS>(fin, fout, nullptr, p, x, y, z, nullptr, seed, !region);
     else
-        lbm_node<T, true, false, CS>(fin, fout, nullptr, p, x, y, z, nullptr, seed, !region);
+        lbm_node<T, true, false, KEEP, CS>(fin, fout, nullptr, p, x, y, z, nullptr, seed, !region);
 }
 
 // The force region's nodes in rows of 128 along x over the whole lattice (the
 // far field's layout: y and z uniform over a block); threads outside the
 // region return at once. Cheaper per node than the list form when the region
 // is a large part of the lattice.
-template <class T, bool CS = true>
+template <class T, bool KEEP, bool CS = true>
 __global__ void __launch_bounds__(128) k_lbm_near_rows(const T *__restrict__ fin, T *__restrict__ fout,
                                                        float4 *__restrict__ F, LbmParams p,
                                                        const unsigned *__restrict__ bits, float4 *__restrict__ vel,
@@ -638,12 +639,12 @@ __global__ void __launch_bounds__(128) k_lbm_near_rows(const T *__restrict__ fin
     if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *seed_out = seed + 1u;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.nx) return;
-    const int y = blockIdx.y, z = plane_of(p, blockIdx.z);
+    const int y = blockIdx.y, z = plane_of<KEEP || !CS>(p, blockIdx.z);
     if (!region_has(bits, tile_index(p, x >> p.tlx, y >> p.tly, z >> p.tlz))) return;
     if (y > 0 && y < p.ny - 1)
-        lbm_node<T, false, true, CS>(fin, fout, F, p, x, y, z, vel, seed);
+        lbm_node<T, false, true, KEEP, CS>(fin, fout, F, p, x, y, z, vel, seed);
     else
-        lbm_node<T, true, true, CS>(fin, fout, F, p, x, y, z, vel, seed);
+        lbm_node<T, true, true, KEEP, CS>(fin, fout, F, p, x, y, z, vel, seed);
 }
 
 // The force region's tiles, with the force field; also stores u(t) there.
@@ -653,7 +654,7 @@ __global__ void __launch_bounds__(128) k_lbm_near_rows(const T *__restrict__ fin
 // the running count of set bits before each bitset word (nwords + 1
 // entries); the k-th tile of the region is then found by a binary search
 // over those counts and a scan of one word.
-template <class T, bool CS = true>
+template <class T, bool KEEP, bool CS = true>
 __global__ void __launch_bounds__(kTileBlock, 8) k_lbm_near(const T *__restrict__ fin, T *__restrict__ fout,
                                                             float4 *__restrict__ F, LbmParams p,
                                                             const unsigned *__restrict__ bits, int nwords,
@@ -662,7 +663,6 @@ __global__ void __launch_bounds__(kTileBlock, 8) k_lbm_near(const T *__restrict_
                                                             unsigned *__restrict__ seed_out) {
     extern __shared__ int before[];  // [nwords + 1]: set bits in the words before word j
     __shared__ int warp_sum[kTileBlock / 32];
-    clear_words(clear, nwords, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
     const unsigned seed = *seed_in;
     if ((blockIdx.x | threadIdx.x) == 0) *seed_out = seed + 1u;
     // running counts: thread i takes a contiguous chunk of words
@@ -703,10 +703,11 @@ __global__ void __launch_bounds__(kTileBlock, 8) k_lbm_near(const T *__restrict_
         int x, y, z;
         if (!tile_node(p, tx, r % p.nty, r / p.nty, (w & 1) * kTileBlock + threadIdx.x, x, y, z)) continue;
         if (y > 0 && y < p.ny - 1)
-            lbm_node<T, false, true, CS>(fin, fout, F, p, x, y, z, vel, seed);
+            lbm_node<T, false, true, KEEP, CS>(fin, fout, F, p, x, y, z, vel, seed);
         else
-            lbm_node<T, true, true, CS>(fin, fout, F, p, x, y, z, vel, seed);
+            lbm_node<T, true, true, KEEP, CS>(fin, fout, F, p, x, y, z, vel, seed);
     }
+    clear_words_list(clear, nwords);
 }
 
 // ---------------------------------------------------------------- pair kernels
@@ -716,7 +717,7 @@ __global__ void __launch_bounds__(kTileBlock, 8) k_lbm_near(const T *__restrict_
 // whole-lattice and far-field forms are held to 72 registers (14 blocks per
 // SM, a 16-byte spill): FP16-SR far field at 128^3 32.9 us against 34.3 us
 // at 80 registers and 34.5 us at 64 (an 84-byte spill).
-template <class T>
+template <class T, bool KEEP>
 __global__ void __launch_bounds__(64, 14) k_lbm_pairs(const T *__restrict__ fin, T *__restrict__ fout, LbmParams p,
                                                   const unsigned *__restrict__ seed_in,
                                                   unsigned *__restrict__ seed_out) {
@@ -724,29 +725,29 @@ __global__ void __launch_bounds__(64, 14) k_lbm_pairs(const T *__restrict__ fin,
     if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *seed_out = seed + 1u;
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (x0 >= p.nx) return;
-    const int y = blockIdx.y, z = plane_of(p, blockIdx.z);
+    const int y = blockIdx.y, z = plane_of<KEEP>(p, blockIdx.z);
     if (y > 0 && y < p.ny - 1)
-        lbm_pair<T, false, false>(fin, fout, nullptr, p, x0, y, z, nullptr, seed);
+        lbm_pair<T, false, false, KEEP>(fin, fout, nullptr, p, x0, y, z, nullptr, seed);
     else
-        lbm_pair<T, true, false>(fin, fout, nullptr, p, x0, y, z, nullptr, seed);
+        lbm_pair<T, true, false, KEEP>(fin, fout, nullptr, p, x0, y, z, nullptr, seed);
 }
 
-template <class T>
+template <class T, bool KEEP>
 __global__ void __launch_bounds__(64, 14) k_lbm_far_pairs(const T *__restrict__ fin, T *__restrict__ fout, LbmParams p,
                                                       const unsigned *__restrict__ bits,
                                                       const unsigned *__restrict__ seed_in) {
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (x0 >= p.nx) return;
-    const int y = blockIdx.y, z = plane_of(p, blockIdx.z);
+    const int y = blockIdx.y, z = plane_of<KEEP>(p, blockIdx.z);
     if (region_has(bits, tile_index(p, x0 >> p.tlx, y >> p.tly, z >> p.tlz))) return;
     const unsigned seed = *seed_in;
     if (y > 0 && y < p.ny - 1)
-        lbm_pair<T, false, false>(fin, fout, nullptr, p, x0, y, z, nullptr, seed);
+        lbm_pair<T, false, false, KEEP>(fin, fout, nullptr, p, x0, y, z, nullptr, seed);
     else
-        lbm_pair<T, true, false>(fin, fout, nullptr, p, x0, y, z, nullptr, seed);
+        lbm_pair<T, true, false, KEEP>(fin, fout, nullptr, p, x0, y, z, nullptr, seed);
 }
 
-template <class T>
+template <class T, bool KEEP>
 __global__ void __launch_bounds__(64) k_lbm_near_pairs(const T *__restrict__ fin, T *__restrict__ fout,
                                                        float4 *__restrict__ F, LbmParams p,
                                                        const unsigned *__restrict__ bits, float4 *__restrict__ vel,
@@ -757,12 +758,12 @@ __global__ void __launch_bounds__(64) k_lbm_near_pairs(const T *__restrict__ fin
     if ((blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *seed_out = seed + 1u;
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (x0 >= p.nx) return;
-    const int y = blockIdx.y, z = plane_of(p, blockIdx.z);
+    const int y = blockIdx.y, z = plane_of<KEEP>(p, blockIdx.z);
     if (!region_has(bits, tile_index(p, x0 >> p.tlx, y >> p.tly, z >> p.tlz))) return;
     if (y > 0 && y < p.ny - 1)
-        lbm_pair<T, false, true>(fin, fout, F, p, x0, y, z, vel, seed);
+        lbm_pair<T, false, true, KEEP>(fin, fout, F, p, x0, y, z, vel, seed);
     else
-        lbm_pair<T, true, true>(fin, fout, F, p, x0, y, z, vel, seed);
+        lbm_pair<T, true, true, KEEP>(fin, fout, F, p, x0, y, z, vel, seed);
 }
 
 // Grid of the pair kernels: up to 64 pairs per block along x.
@@ -770,6 +771,12 @@ static dim3 pair_grid(const LbmParams &p, int &bx) {
     const int pairs = p.nx / 2;
     bx = pairs < 64 ? pairs : 64;
     return dim3((pairs + bx - 1) / bx, p.ny, p.nz);
+}
+
+// Grid of the one-node row kernels: up to 128 nodes per block along x.
+static dim3 row_grid(const LbmParams &p, int &bx) {
+    bx = p.nx < 128 ? p.nx : 128;
+    return dim3((p.nx + bx - 1) / bx, p.ny, p.nz);
 }
 
 // The pair form applies to 16-bit storage with nx even, when the launch
@@ -826,94 +833,99 @@ __global__ void k_macro(const T *__restrict__ f, const float4 *__restrict__ F, L
 // ---------------------------------------------------------------- launchers
 size_t pop_bytes(int fmt) { return fmt == POP_F32 ? 4 : 2; }
 
-template <class T>
-static cudaError_t lbm_t(const void *fin, void *fout, const LbmParams &p, const unsigned *seed, unsigned *next_seed,
+template <class T, bool KEEP>
+static cudaError_t lbm_t(const T *fin, T *fout, const LbmParams &p, const unsigned *seed, unsigned *next_seed,
                          cudaStream_t s) {
+    int bx;
     if constexpr (sizeof(T) == 2) {
         if (use_pairs<T>(p)) {
-            int bx;
             const dim3 grid = pair_grid(p, bx);
-            k_lbm_pairs<T><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), p, seed, next_seed);
+            k_lbm_pairs<T, KEEP><<<grid, bx, 0, s>>>(fin, fout, p, seed, next_seed);
             return cudaGetLastError();
         }
     }
-    const int bx = p.nx < 128 ? p.nx : 128;
-    dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
-    k_lbm<T><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), p, seed, next_seed);
+    const dim3 grid = row_grid(p, bx);
+    k_lbm<T, KEEP><<<grid, bx, 0, s>>>(fin, fout, p, seed, next_seed);
     return cudaGetLastError();
 }
 
-template <class T>
-static cudaError_t far_t(const void *fin, void *fout, const LbmParams &p, const unsigned *bits, const unsigned *seed,
+template <class T, bool KEEP>
+static cudaError_t far_t(const T *fin, T *fout, const LbmParams &p, const unsigned *bits, const unsigned *seed,
                          bool spec, cudaStream_t s) {
+    int bx;
     if constexpr (sizeof(T) == 2) {
         if (use_pairs<T>(p)) {
-            int bx;
             const dim3 grid = pair_grid(p, bx);
-            k_lbm_far_pairs<T><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), p, bits, seed);
+            k_lbm_far_pairs<T, KEEP><<<grid, bx, 0, s>>>(fin, fout, p, bits, seed);
             return cudaGetLastError();
         }
     }
-    const int bx = p.nx < 128 ? p.nx : 128;
-    dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
+    const dim3 grid = row_grid(p, bx);
     if constexpr (std::is_same<T, float>::value) {
         if (p.l2) {  // L2-normal form (FP32 only)
             if (spec)
-                k_lbm_far<T, true, false><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), p,
-                                                              bits, seed);
+                k_lbm_far<T, true, false, false><<<grid, bx, 0, s>>>(fin, fout, p, bits, seed);
             else
-                k_lbm_far<T, false, false><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), p,
-                                                               bits, seed);
+                k_lbm_far<T, false, false, false><<<grid, bx, 0, s>>>(fin, fout, p, bits, seed);
             return cudaGetLastError();
         }
     }
     if (spec)
-        k_lbm_far<T, true><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), p, bits, seed);
+        k_lbm_far<T, true, KEEP><<<grid, bx, 0, s>>>(fin, fout, p, bits, seed);
     else
-        k_lbm_far<T, false><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), p, bits, seed);
+        k_lbm_far<T, false, KEEP><<<grid, bx, 0, s>>>(fin, fout, p, bits, seed);
     return cudaGetLastError();
 }
 
-template <class T>
-static cudaError_t near_t(const void *fin, void *fout, float4 *F, const LbmParams &p, const unsigned *bits,
-                          float4 *vel, int blocks, const unsigned *seed, unsigned *next_seed, unsigned *clear,
-                          cudaStream_t s) {
+template <class T, bool KEEP>
+static cudaError_t near_t(const T *fin, T *fout, float4 *F, const LbmParams &p, const unsigned *bits, float4 *vel,
+                          int blocks, const unsigned *seed, unsigned *next_seed, unsigned *clear, cudaStream_t s) {
     const int nwords = (int)(((long long)p.ntx * p.nty * p.ntz + 31) / 32);
     const size_t smem = sizeof(int) * ((size_t)nwords + 1);
+    int bx;
     if constexpr (std::is_same<T, float>::value) {
         if (p.l2) {  // L2-normal form (FP32 only)
             if (blocks <= 0) {
-                const int bx = p.nx < 128 ? p.nx : 128;
-                dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
-                k_lbm_near_rows<T, false><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), F, p,
-                                                              bits, vel, seed, clear, nwords, next_seed);
+                const dim3 grid = row_grid(p, bx);
+                k_lbm_near_rows<T, false, false><<<grid, bx, 0, s>>>(fin, fout, F, p, bits, vel, seed, clear, nwords,
+                                                                     next_seed);
             } else {
-                k_lbm_near<T, false><<<blocks, kTileBlock, smem, s>>>(static_cast<const T *>(fin),
-                                                                      static_cast<T *>(fout), F, p, bits, nwords, vel,
-                                                                      seed, clear, next_seed);
+                k_lbm_near<T, false, false><<<blocks, kTileBlock, smem, s>>>(fin, fout, F, p, bits, nwords, vel, seed,
+                                                                             clear, next_seed);
             }
             return cudaGetLastError();
         }
     }
     if constexpr (sizeof(T) == 2) {
         if (blocks <= 0 && use_pairs<T>(p)) {  // rows over the whole lattice, two nodes per thread
-            int bx;
             const dim3 grid = pair_grid(p, bx);
-            k_lbm_near_pairs<T><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), F, p, bits,
-                                                     vel, seed, clear, nwords, next_seed);
+            k_lbm_near_pairs<T, KEEP><<<grid, bx, 0, s>>>(fin, fout, F, p, bits, vel, seed, clear, nwords, next_seed);
             return cudaGetLastError();
         }
     }
     if (blocks <= 0) {  // rows over the whole lattice
-        const int bx = p.nx < 128 ? p.nx : 128;
-        dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
-        k_lbm_near_rows<T><<<grid, bx, 0, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), F, p, bits, vel,
-                                               seed, clear, nwords, next_seed);
+        const dim3 grid = row_grid(p, bx);
+        k_lbm_near_rows<T, KEEP><<<grid, bx, 0, s>>>(fin, fout, F, p, bits, vel, seed, clear, nwords, next_seed);
         return cudaGetLastError();
     }
-    k_lbm_near<T><<<blocks, kTileBlock, smem, s>>>(static_cast<const T *>(fin), static_cast<T *>(fout), F, p, bits,
-                                                   nwords, vel, seed, clear, next_seed);
+    k_lbm_near<T, KEEP><<<blocks, kTileBlock, smem, s>>>(fin, fout, F, p, bits, nwords, vel, seed, clear, next_seed);
     return cudaGetLastError();
+}
+
+// f(population pointers, KEEP) for the lattice's storage format.
+template <class Fn>
+static cudaError_t by_format(const void *fin, void *fout, const LbmParams &p, Fn f) {
+    auto typed = [&](auto zero) {
+        using T = decltype(zero);
+        const T *in = static_cast<const T *>(fin);
+        T *out = static_cast<T *>(fout);
+        return p.turn ? f(in, out, std::true_type{}) : f(in, out, std::false_type{});
+    };
+    switch (p.fmt) {
+        case POP_F16: return typed(__half{});
+        case POP_BF16: return typed(__nv_bfloat16{});
+        default: return typed(float{});
+    }
 }
 
 // Every list-form near-field kernel may take up to 4 (max_words + 1) bytes
@@ -922,47 +934,51 @@ cudaError_t prepare_near_field(long long max_words) {
     const int smem = (int)(sizeof(int) * (max_words + 1));
     if (smem <= 48 * 1024) return cudaSuccess;
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(k_lbm_near<float, true>, a, smem);
+    cudaError_t e = cudaFuncSetAttribute(k_lbm_near<float, false, false>, a, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lbm_near<float, false>, a, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lbm_near<float, true>, a, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lbm_near<__half, false>, a, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lbm_near<__half, true>, a, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lbm_near<__nv_bfloat16, false>, a, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_lbm_near<__nv_bfloat16, true>, a, smem);
     return e;
 }
 
+template <class T, bool KEEP>
+static bool is_far_t(const void *fn) {
+    if constexpr (sizeof(T) == 2)
+        if (fn == (const void *)k_lbm_far_pairs<T, KEEP>) return true;
+    return fn == (const void *)k_lbm_far<T, false, KEEP> || fn == (const void *)k_lbm_far<T, true, KEEP>;
+}
+
 bool is_lbm_far_kernel(const void *fn) {
-    return fn == (const void *)k_lbm_far_pairs<__half> || fn == (const void *)k_lbm_far_pairs<__nv_bfloat16> ||
-           fn == (const void *)k_lbm_far<float, false, false> || fn == (const void *)k_lbm_far<float, true, false> ||
-           fn == (const void *)k_lbm_far<float, false> || fn == (const void *)k_lbm_far<__half, false> ||
-           fn == (const void *)k_lbm_far<__nv_bfloat16, false> || fn == (const void *)k_lbm_far<float, true> ||
-           fn == (const void *)k_lbm_far<__half, true> || fn == (const void *)k_lbm_far<__nv_bfloat16, true>;
+    return is_far_t<float, false>(fn) || is_far_t<float, true>(fn) || is_far_t<__half, false>(fn) ||
+           is_far_t<__half, true>(fn) || is_far_t<__nv_bfloat16, false>(fn) || is_far_t<__nv_bfloat16, true>(fn) ||
+           fn == (const void *)k_lbm_far<float, false, false, false> ||
+           fn == (const void *)k_lbm_far<float, true, false, false>;
 }
 
 cudaError_t launch_lbm(const void *fin, void *fout, const LbmParams &p, const unsigned *seed, unsigned *next_seed,
                        cudaStream_t s) {
-    switch (p.fmt) {
-        case POP_F16: return lbm_t<__half>(fin, fout, p, seed, next_seed, s);
-        case POP_BF16: return lbm_t<__nv_bfloat16>(fin, fout, p, seed, next_seed, s);
-        default: return lbm_t<float>(fin, fout, p, seed, next_seed, s);
-    }
+    return by_format(fin, fout, p, [&](auto *in, auto *out, auto keep) {
+        return lbm_t<std::remove_pointer_t<decltype(out)>, decltype(keep)::value>(in, out, p, seed, next_seed, s);
+    });
 }
 
 cudaError_t launch_lbm_far(const void *fin, void *fout, const LbmParams &p, const unsigned *bits,
                            const unsigned *seed, bool spec, cudaStream_t s) {
-    switch (p.fmt) {
-        case POP_F16: return far_t<__half>(fin, fout, p, bits, seed, spec, s);
-        case POP_BF16: return far_t<__nv_bfloat16>(fin, fout, p, bits, seed, spec, s);
-        default: return far_t<float>(fin, fout, p, bits, seed, spec, s);
-    }
+    return by_format(fin, fout, p, [&](auto *in, auto *out, auto keep) {
+        return far_t<std::remove_pointer_t<decltype(out)>, decltype(keep)::value>(in, out, p, bits, seed, spec, s);
+    });
 }
 
 cudaError_t launch_lbm_near(const void *fin, void *fout, float4 *F, const LbmParams &p, const unsigned *bits,
                             float4 *vel, int blocks, const unsigned *seed, unsigned *next_seed, unsigned *clear,
                             cudaStream_t s) {
-    switch (p.fmt) {
-        case POP_F16: return near_t<__half>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, clear, s);
-        case POP_BF16: return near_t<__nv_bfloat16>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, clear, s);
-        default: return near_t<float>(fin, fout, F, p, bits, vel, blocks, seed, next_seed, clear, s);
-    }
+    return by_format(fin, fout, p, [&](auto *in, auto *out, auto keep) {
+        return near_t<std::remove_pointer_t<decltype(out)>, decltype(keep)::value>(in, out, F, p, bits, vel, blocks,
+                                                                                   seed, next_seed, clear, s);
+    });
 }
 
 cudaError_t launch_lbm_init(void *f, const LbmParams &p, cudaStream_t s) {

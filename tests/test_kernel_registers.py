@@ -1,4 +1,4 @@
-"""CPU: the force kernels' register budgets, as the compiler reports them. They
+"""CPU: the register budgets of the force and near-field kernels, as the compiler reports them. They
 are bound by latency and issue, so what a change of the shared stress code
 spills shows in their times; the limits are what they were tuned with."""
 import os
@@ -12,6 +12,7 @@ from paper_2003_03130_gb300 import build
 # source, kernel, registers, bytes of spill stores
 LIMITS = [("tet_force.cu", "k_tet_force", 40, 28), ("chain.cu", "k_cell_chain<2>", 64, 32), ("chain.cu", "k_cell_chain<4>", 64, 44),
           ("relax.cu", "k_relax_cells", 64, 0), ("relax.cu", "k_relax_reverse", 128, 0)]
+LIMITS += [("lbm.cu", f"k_lbm_near<{t}, {keep}, true>", 64, 0) for t in ("float", "__half", "__nv_bfloat16") for keep in ("false", "true")]
 
 
 def used(source):
