@@ -423,11 +423,14 @@ cf_status cf_tape_generation(cf_ctx *ctx, int64_t *out);
 
 /* Reverse the most recent recorded cf_relax call not yet reversed: dF[ncells]
  * is dL/dF for the plate forces at the end of that call. Adds the call's
- * contribution to dL/d(mu, kappa, w) per cell (accumulated in double) and
- * carries dL/dy back to its start (recomputing positions from the
- * checkpoints). Reverse the calls last to first. CF_ESTATE if the tape is
- * empty, or if some cell's material differs from the one the recorded call
- * ran with (the reverse pass would differentiate another forward). */
+ * contribution to dL/d(mu, kappa, w) per cell (per tet in FP32, as the forces;
+ * summed as float pairs of about 48 bits over a warp or a thread block, in
+ * double over blocks and calls) and carries dL/dy back to its start
+ * (recomputing positions from the checkpoints). Reverse the calls last to
+ * first. CF_ENONFINITE if a vector-Jacobian product leaves FP32's range,
+ * CF_ESTATE if the tape is empty, or if some cell's material differs from the
+ * one the recorded call ran with (the reverse pass would differentiate another
+ * forward). */
 cf_status cf_relax_adjoint(cf_ctx *ctx, const double *dF);
 
 /* Accumulated dL/d(mu, kappa, w) per cell, out[ncells][3]. */
@@ -440,7 +443,8 @@ cf_status cf_adjoint_gradients(cf_ctx *ctx, double *out);
 cf_status cf_force_jvp(cf_ctx *ctx, const double *v, double *out);
 
 /* lambda . df/d(mu, kappa, w) per cell for lambda[V][3] at the current
- * positions, out[ncells][3] (double). */
+ * positions, out[ncells][3]; summed as in cf_relax_adjoint. lambda is rounded
+ * to FP32; its scale may be anywhere in FP32's range. */
 cf_status cf_force_param_vjp(cf_ctx *ctx, const double *lambda, double *out);
 
 /* Number of vertices / tets of a cell (0 if the id is unknown). */

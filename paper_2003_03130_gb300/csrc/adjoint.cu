@@ -15,10 +15,13 @@
 //   lambda_y <- lambda_y + dt (J_el + J_plate) m,  lambda_v <- c m,
 //   dL/dtheta += dt m . df/dtheta.
 // J_el = -Hessian of the elastic energy is symmetric, so J_el m is the
-// directional derivative of the forces along m: k_tet_jvp runs the force
-// evaluation of mr.cuh on dual numbers. The forces are linear in
-// (mu_1, mu_2, kappa), so m . df/d(mu, kappa, w) comes from the rates of the
-// unit-modulus energies along m (mr_energy_rates), summed to 48 bits or more.
+// directional derivative of the forces along m: k_tet_jvp evaluates the stress
+// on dual numbers (mr_stress in mr.cuh, the expressions of the force kernels'
+// mr_stress_inv in fused multiply-adds; the two are separate sources). The
+// forces are linear in (mu_1, mu_2, kappa), so m . df/d(mu, kappa, w) comes from
+// the rates of the unit-modulus energies along m (mr_energy_rates): FP32 per
+// tet, as the stress, summed as float pairs of about 48 bits over a warp (on
+// chip, over a thread's tets and steps and the block), FP64 from there.
 #include "plate_ops.cuh"
 
 namespace cf {
@@ -40,56 +43,68 @@ __device__ __forceinline__ void warp_cell_add(int c, double val, double *dst, in
 }
 
 // Add one tet per thread, g = lambda . df/d(mu1, mu2, kappa) of cell c (c < 0:
-// none), to its cell's gradient. Every thread of the block calls. Where the
-// block has one cell (the common case: a cell's tets are contiguous) its
-// threads are summed first, as float pairs (Sum2), and one goes on in FP64:
-// one addition per warp to a single cell's three sums took 35 us for 201 k tets
+// none), times 2^(127 - b) (see direction_exponent), to its cell's gradient.
+// Every thread of the block calls. Where the block has one cell (the common
+// case: a cell's tets are contiguous) the lanes of a warp are summed as float
+// pairs (Sum2), on the warp's largest b, and one thread goes on in FP64: one
+// addition per warp to a single cell's three sums took 35 us for 201 k tets
 // (6 k additions to the same address).
 constexpr int kVjpBlock = 128;
 
-__device__ __forceinline__ void block_add_moduli(const MeshView &m, int c, const float (&g)[3], double scale,
+__device__ __forceinline__ void block_add_moduli(const MeshView &m, int c, const float (&g)[3], int b, double scale,
                                                  double *grad) {
     constexpr int kWarps = kVjpBlock / 32;
     __shared__ Sum2 part[3][kWarps];
-    __shared__ int c0;
+    __shared__ int exponent[kWarps], c0;
     if (threadIdx.x == 0) c0 = c;  // the block's first tet: no later one has an element if it has none
     __syncthreads();
     if (__syncthreads_and(c == c0 || c < 0)) {
-        const int lane = threadIdx.x & 31;
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        const int top = __reduce_max_sync(0xffffffffu, c < 0 ? 1 : b), less = 127 + b - top;
+        const float f = less > 0 ? power_of_two(less) : 0.f;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             Sum2 a;
-            a.hi = c < 0 ? 0.f : g[k];
+            a.hi = c < 0 ? 0.f : f * g[k];
             warp_sum(a);
-            if (lane == 0) part[k][threadIdx.x >> 5] = a;
+            if (lane == 0) part[k][w] = a;
         }
+        if (lane == 0) exponent[w] = top;
         __syncthreads();
         if (threadIdx.x >= 32 || c0 < 0) return;
-        Sum2 a;  // lane k: sum k over the warps
+        double G = 0.0;  // lane k: sum k over the warps
         if (lane < 3)
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                a.add(part[lane][w].hi);
-                a.lo = __fadd_rn(a.lo, part[lane][w].lo);
-            }
-        const double G = a.value(), G0 = __shfl_sync(0xffffffffu, G, 0), G1 = __shfl_sync(0xffffffffu, G, 1);
+            for (int q = 0; q < kWarps; ++q) G += part[lane][q].value() * power_of_two_64(exponent[q]);
+        const double G0 = __shfl_sync(0xffffffffu, G, 0), G1 = __shfl_sync(0xffffffffu, G, 1);
         if (lane < 3) add_moduli_rate(lane, G0, G1, G, __ldg(m.mat + c0), scale, grad + 3 * c0);
     } else if (c >= 0) {
         const float4 mat = __ldg(m.mat + c);
+        const double s = scale * power_of_two_64(b);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-            add_moduli_rate(k, (double)g[0], (double)g[1], (double)g[2], mat, scale, grad + 3 * c);
+            add_moduli_rate(k, (double)g[0], (double)g[1], (double)g[2], mat, s, grad + 3 * c);
     }
+}
+
+// Gradient dH of a direction on tet a4, times 2^(127 - b); returns b.
+__device__ __forceinline__ int scaled_grad(const float4 *__restrict__ v, int4 a4, const float (&Bm)[3][3],
+                                           float (&dH)[3][3]) {
+    const float4 l0 = __ldg(v + a4.x), l1 = __ldg(v + a4.y), l2 = __ldg(v + a4.z), l3 = __ldg(v + a4.w);
+    const int b = direction_exponent(largest(l0, largest(l1, largest(l2, largest(l3, 0.f)))));
+    const float f = power_of_two(254 - b);
+    tet_grad(times(l0, f), times(l1, f), times(l2, f), times(l3, f), Bm, dH);
+    return b;
 }
 
 // lambda . df/d(mu, kappa, w) per cell, times `scale`, added into grad[3 c + .]:
 // the rates of the unit-modulus energies along lambda's gradient
 // (mr_energy_rates). Three stresses and 36 FP64 products per tet in its place
-// were bound by FP64: 201 k tets 53 us, now 9.9; 20 k tets 12.2 us, now 5.9.
+// were bound by FP64: 201 k tets 52 us, now 10.9 (9.7 without the
+// directions' scaling); 20 k tets 12.0 us, now 7.0.
 __global__ void __launch_bounds__(kVjpBlock) k_param_vjp(MeshView m, const float4 *__restrict__ u,
                                                    const float4 *__restrict__ lam, double scale, double *grad) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    int c = -1;
+    int c = -1, b = 1;
     float g[3] = {0.f, 0.f, 0.f};
     if (t < m.T) {
         const int4 a4 = __ldg(m.tet + t);
@@ -97,7 +112,7 @@ __global__ void __launch_bounds__(kVjpBlock) k_param_vjp(MeshView m, const float
         load_B(m, t, Bm);
         float H[3][3], dH[3][3];
         tet_grad(__ldg(u + a4.x), __ldg(u + a4.y), __ldg(u + a4.z), __ldg(u + a4.w), Bm, H);
-        tet_grad(__ldg(lam + a4.x), __ldg(lam + a4.y), __ldg(lam + a4.z), __ldg(lam + a4.w), Bm, dH);
+        b = scaled_grad(lam, a4, Bm, dH);
         InvT<float> inv;
         invariants_t(H, inv);
         mr_energy_rates(H, dH, inv, g);
@@ -106,7 +121,7 @@ __global__ void __launch_bounds__(kVjpBlock) k_param_vjp(MeshView m, const float
         for (int k = 0; k < 3; ++k) g[k] *= -V0;
         c = __ldg(m.tcell + t);
     }
-    block_add_moduli(m, c, g, scale, grad);
+    block_add_moduli(m, c, g, b, scale, grad);
 }
 
 cudaError_t launch_param_vjp(const MeshView &m, const float4 *u, const float4 *lam, double scale, double *grad,
@@ -120,13 +135,15 @@ cudaError_t launch_param_vjp(const MeshView &m, const float4 *u, const float4 *l
 // Corner tangents d f / d eps of f(u + eps v) into m.fc. GRAD: the same
 // evaluation also adds v . df/d(mu, kappa, w), times `scale`, to grad: the
 // reverse step needs both along the same direction (528 k tets: 31 us, where
-// two launches took 20 + 126 us). Bound by its ~900 FP32 operations a tet.
+// two launches took 20 + 126 us). Bound by its ~900 FP32 operations a tet;
+// held to 72 registers (20 bytes of spills): a recomputed and reversed step of
+// 872 k tets 111 us, 115 at 80 registers and 121 at the 96 it would take.
 template <bool GRAD>
-__global__ void __launch_bounds__(GRAD ? kVjpBlock : 128) k_tet_jvp(MeshView m, const float4 *__restrict__ u,
+__global__ void __launch_bounds__(GRAD ? kVjpBlock : 128, GRAD ? 7 : 0) k_tet_jvp(MeshView m, const float4 *__restrict__ u,
                                                  const float4 *__restrict__ v, double scale, double *grad) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (!GRAD && t >= m.T) return;
-    int c = -1;
+    int c = -1, b = 1;
     float g[3] = {0.f, 0.f, 0.f};
     if (t < m.T) {
         const int4 a4 = __ldg(m.tet + t);
@@ -134,7 +151,10 @@ __global__ void __launch_bounds__(GRAD ? kVjpBlock : 128) k_tet_jvp(MeshView m, 
         load_B(m, t, Bm);
         float H[3][3], dH[3][3];
         tet_grad(__ldg(u + a4.x), __ldg(u + a4.y), __ldg(u + a4.z), __ldg(u + a4.w), Bm, H);
-        tet_grad(__ldg(v + a4.x), __ldg(v + a4.y), __ldg(v + a4.z), __ldg(v + a4.w), Bm, dH);
+        if (GRAD)
+            b = scaled_grad(v, a4, Bm, dH);
+        else
+            tet_grad(__ldg(v + a4.x), __ldg(v + a4.y), __ldg(v + a4.z), __ldg(v + a4.w), Bm, dH);
         const float4 mat = __ldg(m.mat + mat_slot(m, t));
         const float V0 = __ldg(m.V0 + t);
         float f[4][3];
@@ -147,9 +167,12 @@ __global__ void __launch_bounds__(GRAD ? kVjpBlock : 128) k_tet_jvp(MeshView m, 
             c = __ldg(m.tcell + t);
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a) m.fc[a * m.T + t] = make_float4(f[a][0], f[a][1], f[a][2], 0.f);
+        for (int a = 0; a < 4; ++a) {
+            const float4 fa = make_float4(f[a][0], f[a][1], f[a][2], 0.f);
+            m.fc[a * m.T + t] = GRAD ? times(fa, power_of_two(b)) : fa;
+        }
     }
-    if (GRAD) block_add_moduli(m, c, g, scale, grad);
+    if (GRAD) block_add_moduli(m, c, g, b, scale, grad);
 }
 
 cudaError_t launch_force_jvp(const MeshView &m, const float4 *u, const float4 *v, float4 *out, unsigned *err,

@@ -218,42 +218,66 @@ __device__ __forceinline__ void mr_stress(const Dual (&H)[3][3], float mu1, floa
         }
 }
 
+// x / 3, to within an ulp: a factor 1.f / 3.f would be off by the same 3e-8 in
+// every tet.
+__device__ __forceinline__ float third(float x) {
+    const float c = 1.f / 3.f, y = x * c;
+    return fmaf(fmaf(-3.f, y, x), c, y);
+}
+
 // Rates of the three unit-modulus energies of one tet along dH: g = d/d eps of
 // (I - 3)/2, (K - 3)/2 and (J - 1)^2/2 at H + eps dH, so that a direction
 // lambda of the vertices with dH its gradient has lambda . f = -V0 g . (mu1,
 // mu2, kappa). One contraction per modulus takes the place of a stress and
-// twelve force components per modulus. With de = 2 (tr dH + H:dH) and
-// dj = tr dH + dj2, dj2 = t tr dH - tr(H dH) + cof(H):dH, the O(|dH|) parts
-// of de - 2 dj cancel by hand (J de - 2 dj = 2 (H:dH - dj2) + j de, and twice
-// that for K), so every term left is O(|H| |dH|), as in the stress:
+// twelve force components per modulus. With hd = H:dH and
+// r = (H + H^T - t I - cof(H)):dH, de = 2 (tr dH + hd) and
+// dj = tr dH + hd - r, and the O(|dH|) parts of de - 2 dj cancel by hand
+// (J de - 2 dj = 2 r + j de, and twice that for K), so every term left is
+// O(|H| |dH|), as in the stress; r is summed from the differences, which
+// vanish under a rotation, not as the difference of two sums:
 //   d(I) = s/J [J de - 2/3 (3 + e) dj],  s = J^-2/3,
 //   d(K) = s^2/J [J dK' - 4/3 K' dj],    K' = 3 + 2e + (e^2 - q)/2.
+// Sums over a cell against 64 bits, beside FP64 products of lambda with the
+// forces of three unit-modulus stresses in its place: 0.9 of their error over
+// random directions (noise, stretched, squashed and rotated cells of 1.7 k to
+// 20 k tets; 0.8 to 1.25 for smooth directions).
 __device__ __forceinline__ void mr_energy_rates(const float (&H)[3][3], const float (&dH)[3][3], const InvT<float> &v,
                                                 float (&g)[3]) {
     const float dt = dH[0][0] + dH[1][1] + dH[2][2];
-    float hd = 0.f, hx = 0.f, eg = 0.f;  // H:dH, tr(H dH), E:(F^T dH)
+    float hd = 0.f, r = 0.f, eg = 0.f;  // eg = E:(F^T dH)
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
+            const int i1 = (i + 1) % 3, i2 = (i + 2) % 3, k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+            const float sym = i == k ? H[i][k] + H[k][i] - v.t : H[i][k] + H[k][i];
+            r += (sym - fmaf(H[i1][k1], H[i2][k2], -(H[i1][k2] * H[i2][k1]))) * dH[i][k];
             hd += H[i][k] * dH[i][k];
-            hx += H[i][k] * dH[k][i];
             eg += v.E[i][k] * (dH[i][k] + H[0][i] * dH[0][k] + H[1][i] * dH[1][k] + H[2][i] * dH[2][k]);
         }
-    const float ddet = (H[1][1] * H[2][2] - H[1][2] * H[2][1]) * dH[0][0] + (H[1][2] * H[2][0] - H[1][0] * H[2][2]) * dH[0][1] +
-                       (H[1][0] * H[2][1] - H[1][1] * H[2][0]) * dH[0][2] + (H[0][2] * H[2][1] - H[0][1] * H[2][2]) * dH[1][0] +
-                       (H[0][0] * H[2][2] - H[0][2] * H[2][0]) * dH[1][1] + (H[0][1] * H[2][0] - H[0][0] * H[2][1]) * dH[1][2] +
-                       (H[0][1] * H[1][2] - H[0][2] * H[1][1]) * dH[2][0] + (H[0][2] * H[1][0] - H[0][0] * H[1][2]) * dH[2][1] +
-                       (H[0][0] * H[1][1] - H[0][1] * H[1][0]) * dH[2][2];
-    const float dj2 = v.t * dt - hx + ddet;
-    const float dj = dt + dj2, de = 2.f * (dt + hd), r = hd - dj2;
+    const float dj = dt + (hd - r), de = 2.f * (dt + hd);
     const float dk = v.e * de - 2.f * eg;  // dK' - 2 de, with dq = 4 E:(F^T dH)
     const float k3 = 2.f * v.e + 0.5f * (v.e * v.e - v.q);
     const float s = expf(-(2.f / 3.f) * v.L), iJ = 1.f / v.J;
-    g[0] = 0.5f * s * iJ * (2.f * r + v.j * de - (2.f / 3.f) * v.e * dj);
-    g[1] = 0.5f * s * s * iJ * (4.f * r + dk + v.j * (2.f * de + dk) - (4.f / 3.f) * k3 * dj);
+    g[0] = third(s * iJ * (3.f * r + 1.5f * v.j * de - v.e * dj));
+    g[1] = third(s * s * iJ * (6.f * r + 1.5f * (dk + v.j * (2.f * de + dk)) - 2.f * k3 * dj));
     g[2] = v.j * dj;
 }
+
+// The rates are linear in dH. Directions are taken times a power of two that
+// brings their largest component x (>= 0) near 1, 2^(127 - b) with b its biased
+// exponent, and the sums back in FP64, so that neither leaves FP32's range
+// where the direction itself does not. Infinities and NaN: factor 1.
+__device__ __forceinline__ int direction_exponent(float x) {
+    const int b = __float_as_int(x) >> 23;
+    return b == 255 ? 127 : min(max(b, 1), 253);
+}
+__device__ __forceinline__ float power_of_two(int b) { return __int_as_float(b << 23); }  // 2^(b - 127), 0 < b < 255
+__device__ __forceinline__ double power_of_two_64(int b) { return __hiloint2double((b - 127 + 1023) << 20, 0); }
+__device__ __forceinline__ float largest(float4 a, float x) {
+    return fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), x));
+}
+__device__ __forceinline__ float4 times(float4 a, float x) { return make_float4(a.x * x, a.y * x, a.z * x, 0.f); }
 
 // A sum of floats kept as an unevaluated pair hi + lo: every addition is the
 // exact two-sum (D. E. Knuth, The Art of Computer Programming vol. 2, 4.2.2),
@@ -267,7 +291,8 @@ struct Sum2 {
         lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)));
         hi = t;
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    // an infinite or NaN sum: lo is NaN by then
+    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
 };
 
 // Sum of a pair over the lanes of a full warp (every lane ends with it).

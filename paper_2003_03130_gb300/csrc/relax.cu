@@ -317,6 +317,7 @@ __global__ void __launch_bounds__(kReverseBlock, 1)
                     unsigned *err) {
     extern __shared__ float4 su[];  // [vertices of the cell] displacements, then m, then the corner tangents
     __shared__ Sum2 part[3][kReverseBlock / 32];
+    __shared__ float warp_top[kReverseBlock / 32];
     const cg::cluster_group cluster = cg::this_cluster();
     const RelaxPart p = pl.parts[blockIdx.x];
     float4 *sm = su + p.cell_nv;
@@ -324,12 +325,24 @@ __global__ void __launch_bounds__(kReverseBlock, 1)
     const int lane = threadIdx.x & 3;
     const float4 mat = __ldg(m.mat + p.cell);
     const PlateZ pz = plates_of(m, p.cell, zlo, zhi);
+    float top = 0.f;
     for (int j = threadIdx.x; j < p.cell_nv; j += kReverseBlock) {
         const int v = p.cell_v0 + j;
         su[j] = __ldg(y + (size_t)(n - 1) * m.V + v);
         const float4 a = ly[v], b = lv[v];
         sm[j] = make_float4(fmaf(dt, a.x, b.x), fmaf(dt, a.y, b.y), fmaf(dt, a.z, b.z), 0.f);
+        top = largest(sm[j], top);
     }
+    // m and the tangents are held times 2^(127 - b), see direction_exponent;
+    // every block of the cluster has read the whole cell, so they agree on b
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    if ((threadIdx.x & 31) == 0) warp_top[threadIdx.x >> 5] = top;
+    __syncthreads();
+    for (int w = 0; w < kReverseBlock / 32; ++w) top = fmaxf(top, warp_top[w]);
+    const int b2 = direction_exponent(top);
+    const float down = power_of_two(254 - b2), up = power_of_two(b2);
+    for (int j = threadIdx.x; j < p.cell_nv; j += kReverseBlock) sm[j] = times(sm[j], down);
     cluster.sync();  // ly, lv are read before any block changes them
     Sum2 g[3];
     for (int step = n - 1; step >= 0; --step) {
@@ -366,10 +379,12 @@ __global__ void __launch_bounds__(kReverseBlock, 1)
             const uint4 e = live ? __ldg(pl.inc + 4 * (size_t)v + lane) : make_uint4(~0u, ~0u, ~0u, ~0u);
             float jx, jy, jz;
             sum_incidences(e, fc, jx, jy, jz);
+            jx *= up, jy *= up, jz *= up;
             float4 a, b, mn = make_float4(0.f, 0.f, 0.f, 0.f);
             if (live) {
                 const float z = __ldg(m.xr + v).z + __ldg(now + v).z;
-                adjoint_move(ly[v], make_float4(jx, jy, jz, 0.f), sm[local], z, pz, dt, c, kp, a, b, mn);
+                adjoint_move(ly[v], make_float4(jx, jy, jz, 0.f), times(sm[local], up), z, pz, dt, c, kp, a, b, mn);
+                mn = times(mn, down);
             }
             if (j0 == 0) cluster.barrier_wait();  // every block is done with the old m
             __syncwarp();                         // the four lanes have read ly
@@ -393,6 +408,7 @@ __global__ void __launch_bounds__(kReverseBlock, 1)
     double G = 0.0;
     if (threadIdx.x < 3)
         for (int w = 0; w < kReverseBlock / 32; ++w) G += part[threadIdx.x][w].value();
+    G *= power_of_two_64(b2);
     const double G0 = __shfl_sync(0xffffffffu, G, 0), G1 = __shfl_sync(0xffffffffu, G, 1);
     if (threadIdx.x < 3) add_moduli_rate(threadIdx.x, G0, G1, G, mat, (double)dt, grad + 3 * p.cell);
 }
