@@ -478,6 +478,7 @@ cf_status cf_lbm_init(cf_ctx *c, int32_t nx, int32_t ny, int32_t nz, double tau,
         return fail(c, CF_EINVAL, "body force must be finite");
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     drop_graphs(c);
+    cf_free_plan(c);
     dfree(c->f[0]);
     dfree(c->f[1]);
     dfree(c->F);
@@ -614,6 +615,7 @@ cf_status cf_mesh_init_batch(cf_ctx *c, int32_t ncells, const int32_t *nv, const
                         cudaGetErrorString(e_));                                                       \
         }                                                                                              \
     } while (0)
+    cf_free_plan(c);  // of the old mesh
     TRY_N(dalloc(&n.xr, V1));
     TRY_N(dalloc(&n.u[0], V1));
     TRY_N(dalloc(&n.u[1], V1));
@@ -1283,7 +1285,7 @@ static cf_status get_macro(cf_ctx *c, double *rho_out, double *u_out) {
     if (!c->lbm_ready) return fail(c, CF_ESTATE, "no fluid: call cf_lbm_init");
     const size_t N = (size_t)c->lp.N;
     double *d;
-    CUDA_TRY(c, dalloc(&d, u_out ? 3 * N : N));
+    CUDA_TRY(c, dalloc_spare(c, &d, u_out ? 3 * N : N));
     // the last step's force region, in the tiling that step ran with
     LbmParams q = c->lp;
     const unsigned *bits = nullptr;

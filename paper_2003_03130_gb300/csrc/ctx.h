@@ -55,6 +55,7 @@ using namespace cf;
 struct cf_ctx;
 // Frees the compression/adjoint buffers and the tape (csrc/plates.cu).
 void cf_free_adjoint(cf_ctx *c);
+void cf_free_plan(cf_ctx *c);  // the on-chip relaxation's; the next relaxation makes it again
 
 struct cf_ctx {
     using CellInfo = cf::CellInfo;
@@ -145,8 +146,9 @@ struct cf_ctx {
     double *grad = nullptr, *gtmp = nullptr, *pforce = nullptr, *dF = nullptr;
     int adj_V = 0, adj_C = 0;
     // on-chip relaxation (csrc/relax.cu): the plan of the current mesh, made
-    // by the first relaxation; plan_state 0: not tried, 1: made, 2: the mesh
-    // does not fit (general path)
+    // by the first relaxation; plan_state 0: not made, 1: made, 2: the mesh
+    // does not fit or is faster in launches. Given back where cells are added,
+    // the lattice is allocated, or a checkpoint or a field finds no memory.
     int plan_state = 0;
     RelaxPlan plan{};
     RelaxPart *plan_parts = nullptr;
@@ -186,6 +188,16 @@ cudaError_t dalloc(T **p, size_t count) {
     *p = nullptr;
     if (count == 0) count = 1;
     return cudaMalloc((void **)p, sizeof(T) * count);
+}
+
+// dalloc at the cost of the on-chip relaxation's plan.
+template <class T>
+cudaError_t dalloc_spare(cf_ctx *c, T **p, size_t count) {
+    const cudaError_t e = dalloc(p, count);
+    if (e != cudaErrorMemoryAllocation || c->plan_state != 1) return e;
+    cudaGetLastError();
+    cf_free_plan(c);
+    return dalloc(p, count);
 }
 
 template <class T>

@@ -13,6 +13,7 @@
 // accumulating dt m . df/d(mu, kappa, w) per cell in double.
 #include <algorithm>
 #include <functional>
+#include <new>
 #include <queue>
 
 #include "ctx.h"
@@ -42,11 +43,7 @@ void free_adjoint(cf_ctx *c) {
     dfree(c->dF);
     dfree(c->zlo);
     dfree(c->zhi);
-    dfree(c->plan_parts);
-    dfree(c->plan_rows);
-    dfree(c->plan_list);
-    dfree(c->plan_inc);
-    c->plan_state = 0;
+    cf_free_plan(c);
     c->adj_V = c->adj_C = 0;
 }
 
@@ -123,6 +120,16 @@ double on_chip_time(const StepTime &q, const std::vector<int> &nt, int slots) {
     return end;
 }
 
+struct PlanScratch {
+    int4 *cells = nullptr;
+    int *counts = nullptr, *slot = nullptr;
+    ~PlanScratch() {
+        dfree(cells);
+        dfree(counts);
+        dfree(slot);
+    }
+};
+
 // The on-chip relaxation's plan for the current mesh, if it fits and is
 // expected to be faster: cells cut into `cs` blocks, the fewest that hold a
 // part in shared memory; more, up to eight, while every block still gets an SM
@@ -133,54 +140,38 @@ double on_chip_time(const StepTime &q, const std::vector<int> &nt, int slots) {
 // on chip against three launches a step: 64 cells of 8.3 k tets 16.3 and 28.9
 // us, reverse steps 47 and 70; 2,000 cells of 192 tets 36.9 and 25.8, reverse
 // 88 and 66; 300 of 192 beside one of 13.6 k 50 and 14.5, reverse 121 and 35.
-cf_status make_plan(cf_ctx *c) {
-    if (c->plan_state) return CF_OK;
-    c->plan_state = 2;
+// plan_state: 1 with the plan, 2 if the mesh takes the launches.
+cudaError_t build_plan(cf_ctx *c) {
     const int C = (int)c->cells.size();
     std::vector<int4> cells(C);
+    c->plan_state = 2;
     for (int k = 0; k < C; ++k) {
         const CellInfo &ci = c->cells[k];
-        if (ci.nv > 0xffff) return CF_OK;
+        if (ci.nv > 0xffff) return cudaSuccess;
         cells[k] = make_int4(ci.v_off, ci.nv, ci.t_off, ci.nt);
     }
-    if (C > INT_MAX / 15) return CF_OK;
+    if (C > INT_MAX / 15) return cudaSuccess;
     int smem = 0;
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
     if (smem <= kRelaxStatic || prepare_relax(smem) != cudaSuccess) {
         cudaGetLastError();
-        return CF_OK;
+        return cudaSuccess;
     }
     const MeshView m = view(c);
-    int4 *d_cells = nullptr;
-    int *d_counts = nullptr, *d_slot = nullptr;
-    auto done = [&](cudaError_t e) {
-        dfree(d_cells);
-        dfree(d_counts);
-        dfree(d_slot);
-        if (c->plan_state != 1) {
-            dfree(c->plan_parts);
-            dfree(c->plan_rows);
-            dfree(c->plan_list);
-            dfree(c->plan_inc);
-        }
-        if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // the general path needs none of it
-        return e == cudaSuccess || e == cudaErrorMemoryAllocation
-                   ? CF_OK
-                   : fail(c, CF_ECUDA, "relaxation plan: %s", cudaGetErrorString(e));
-    };
-#define TRY_P(expr)                               \
-    do {                                          \
-        const cudaError_t e_ = (expr);            \
-        if (e_ != cudaSuccess) return done(e_);   \
+    PlanScratch d;
+#define TRY_P(expr)                                \
+    do {                                           \
+        const cudaError_t e_ = (expr);             \
+        if (e_ != cudaSuccess) return e_;          \
     } while (0)
-    TRY_P(dalloc(&d_cells, C));
-    TRY_P(dalloc(&d_counts, 15 * (size_t)C + 1));
-    TRY_P(cudaMemcpyAsync(d_cells, cells.data(), sizeof(int4) * C, cudaMemcpyHostToDevice, c->stream));
-    TRY_P(launch_relax_count(m, d_cells, C, d_counts, d_counts + 15 * (size_t)C, c->stream));
+    TRY_P(dalloc(&d.cells, C));
+    TRY_P(dalloc(&d.counts, 15 * (size_t)C + 1));
+    TRY_P(cudaMemcpyAsync(d.cells, cells.data(), sizeof(int4) * C, cudaMemcpyHostToDevice, c->stream));
+    TRY_P(launch_relax_count(m, d.cells, C, d.counts, d.counts + 15 * (size_t)C, c->stream));
     std::vector<int> counts(15 * (size_t)C + 1);
-    TRY_P(cudaMemcpyAsync(counts.data(), d_counts, sizeof(int) * counts.size(), cudaMemcpyDeviceToHost, c->stream));
+    TRY_P(cudaMemcpyAsync(counts.data(), d.counts, sizeof(int) * counts.size(), cudaMemcpyDeviceToHost, c->stream));
     TRY_P(cudaStreamSynchronize(c->stream));
-    if (counts.back() > kRelaxDegree) return done(cudaSuccess);
+    if (counts.back() > kRelaxDegree) return cudaSuccess;
     std::vector<int> most_of(C);  // tets of a cell's largest block
     auto largest = [&](int cs, bool &fits) {
         fits = true;
@@ -194,7 +185,7 @@ cf_status make_plan(cf_ctx *c) {
     int cs = 1;
     bool fits = false;
     while (largest(cs, fits), !fits && cs < 8) cs *= 2;
-    if (!fits) return done(cudaSuccess);
+    if (!fits) return cudaSuccess;
     while (cs < 8 && 2LL * cs * C <= c->sms && largest(cs, fits) > kRelaxRound) cs *= 2;
     RelaxPlan pl{};
     pl.cs = cs;
@@ -215,22 +206,22 @@ cf_status make_plan(cf_ctx *c) {
             pl.smem_step = std::max(pl.smem_step, relax_smem(q.cell_nv, q.nv, q.nt, false));
             pl.smem_reverse = std::max(pl.smem_reverse, relax_smem(q.cell_nv, q.nv, q.nt, true));
         }
-    if (nt_all > INT_MAX) return done(cudaSuccess);
+    if (nt_all > INT_MAX) return cudaSuccess;
     pl.NT = (int)nt_all;
     const int slots = relax_clusters(pl);
-    if (slots == 0) return done(cudaSuccess);
+    if (slots == 0) return cudaSuccess;
     largest(cs, fits);
     pl.steps = on_chip_time(kChipStep, most_of, slots) < step_time(kLaunchStep, c->T, c->V);
     pl.reverse = on_chip_time(kChipReverse, most_of, slots) < step_time(kLaunchReverse, c->T, c->V);
-    if (!pl.steps && !pl.reverse) return done(cudaSuccess);
+    if (!pl.steps && !pl.reverse) return cudaSuccess;
     TRY_P(dalloc(&c->plan_parts, parts.size()));
     TRY_P(dalloc(&c->plan_rows, 3 * (size_t)pl.NT));
     TRY_P(dalloc(&c->plan_list, pl.NT));
     TRY_P(dalloc(&c->plan_inc, 4 * (size_t)c->V));
-    TRY_P(dalloc(&d_slot, (size_t)cs * c->T));
+    TRY_P(dalloc(&d.slot, (size_t)cs * c->T));
     TRY_P(cudaMemcpyAsync(c->plan_parts, parts.data(), sizeof(RelaxPart) * parts.size(), cudaMemcpyHostToDevice,
                           c->stream));
-    TRY_P(launch_relax_fill(m, c->plan_parts, pl.nparts, cs, d_cells, c->plan_rows, pl.NT, c->plan_list, d_slot,
+    TRY_P(launch_relax_fill(m, c->plan_parts, pl.nparts, cs, d.cells, c->plan_rows, pl.NT, c->plan_list, d.slot,
                             c->plan_inc, c->stream));
     TRY_P(cudaStreamSynchronize(c->stream));  // the host vectors and the scratch go
 #undef TRY_P
@@ -240,7 +231,27 @@ cf_status make_plan(cf_ctx *c) {
     pl.inc = c->plan_inc;
     c->plan = pl;
     c->plan_state = 1;
-    return done(cudaSuccess);
+    return cudaSuccess;
+}
+
+// Without memory for a plan the launches are taken, and the next call tries
+// again.
+cf_status make_plan(cf_ctx *c) {
+    if (c->plan_state) return CF_OK;
+    cudaError_t e;
+    try {
+        e = build_plan(c);
+    } catch (const std::bad_alloc &) {
+        e = cudaErrorMemoryAllocation;
+    }
+    if (c->plan_state == 1) return CF_OK;
+    const int state = e == cudaSuccess ? c->plan_state : 0;
+    cf_free_plan(c);
+    c->plan_state = state;
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e == cudaSuccess || e == cudaErrorMemoryAllocation
+               ? CF_OK
+               : fail(c, CF_ECUDA, "relaxation plan: %s", cudaGetErrorString(e));
 }
 
 // The plan if the mesh has one that takes steps (reverse: reverse steps) on
@@ -336,7 +347,7 @@ cf_status cf_relax(cf_ctx *c, int32_t n, double dt, double damping, int32_t reco
         for (const CellInfo &ci : c->cells) e.mats.push_back(ci.mat);
         while ((int)c->ckpt.size() < e.ck0 + e.nck) {
             float4 *p = nullptr;
-            CUDA_TRY(c, dalloc(&p, 2 * (size_t)c->V));
+            CUDA_TRY(c, dalloc_spare(c, &p, 2 * (size_t)c->V));
             c->ckpt.push_back(p);
         }
     }
@@ -513,3 +524,11 @@ cf_status cf_force_param_vjp(cf_ctx *c, const double *lam, double *out) {
 }  // extern "C"
 
 void cf_free_adjoint(cf_ctx *c) { free_adjoint(c); }
+
+void cf_free_plan(cf_ctx *c) {
+    dfree(c->plan_parts);
+    dfree(c->plan_rows);
+    dfree(c->plan_list);
+    dfree(c->plan_inc);
+    c->plan_state = 0;
+}
