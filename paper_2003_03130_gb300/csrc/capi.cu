@@ -1342,8 +1342,13 @@ cf_status cf_get_cell_strain(cf_ctx *c, int32_t id, double d_ref, double *out) {
     DeviceGuard dg(c->device);
     unsigned *word = reinterpret_cast<unsigned *>(c->d_status);  // device scratch of the context: two words
     float4 *keep = reinterpret_cast<float4 *>(c->stage);          // and 24 bytes per vertex
-    CUDA_TRY(c, launch_max_extent(view(c), c->u[c->cur], ci->v_off, ci->nv, keep, word, 4 * c->sms, c->stream));
-    CUDA_TRY(c, cudaMemcpyAsync(c->result, word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    if (ci->nv <= kExtentOne) {
+        CUDA_TRY(c, launch_extent_one(view(c), c->u[c->cur], ci->v_off, ci->nv, reinterpret_cast<unsigned *>(c->result),
+                                      c->stream));
+    } else {
+        CUDA_TRY(c, launch_max_extent(view(c), c->u[c->cur], ci->v_off, ci->nv, keep, word, 4 * c->sms, c->stream));
+        CUDA_TRY(c, cudaMemcpyAsync(c->result, word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    }
     const cf_status s = wait_stream(c);
     if (s != CF_OK) return s;
     float d2;

@@ -195,9 +195,13 @@ cudaError_t launch_taylor(const MeshView &m, const float4 *u, int t0, int t1, do
 // depend on the order; the bound is widened by 1e-4, far more than the
 // rounding of the FP32 distances. All pairs of all vertices in one block per
 // tile took 52 us for 4.2 k vertices and 428 us for 37 k; selection and pairs
-// together take 18 and 23 us. Positions enter
-// relative to the cell's integer origin.
-constexpr int kExtentBlock = 256;
+// together take 18 and 23 us. Cells whose pairs of tiles fill at most one
+// round of blocks (8.7 k vertices) take them all without a selection, those of
+// one tile in one block that writes to the host: the whole call for 81 vertices
+// 22 us with the old kernel, 33 with a selection, 15 now; for 365 29, 34
+// and 27, for 4.2 k 68, 41 and 28. Positions enter relative to the cell's
+// integer origin.
+constexpr int kExtentBlock = kExtentOne;
 constexpr int kSelectBlock = 1024;
 
 __device__ __forceinline__ float dist2(float3 a, float3 b) {
@@ -300,12 +304,22 @@ __global__ void __cluster_dims__(kSelectCluster, 1, 1) __launch_bounds__(kSelect
     cg::this_cluster().sync();  // no block leaves while another reads its shared memory
 }
 
-// Pairs of kept vertices, one pair of tiles (row <= column) per block and
-// round; non-negative floats order like their bits.
+// Pairs of kept vertices (KEPT; else of all of the cell's), one pair of tiles
+// (row <= column) per block and round; non-negative floats order like their
+// bits.
+template <bool KEPT>
 __global__ void __launch_bounds__(kExtentBlock) k_extent_pairs(const float4 *__restrict__ keep,
-                                                               const int *__restrict__ nkeep, unsigned *out) {
+                                                               const int *__restrict__ nkeep, MeshView m,
+                                                               const float4 *__restrict__ u, int v0, int nv,
+                                                               unsigned *out) {
     __shared__ float4 tile[kExtentBlock];
-    const int n = *nkeep, nt = (n + kExtentBlock - 1) / kExtentBlock;
+    const int n = KEPT ? *nkeep : nv, nt = (n + kExtentBlock - 1) / kExtentBlock;
+    auto at = [&](int k) {  // padding takes vertex 0: real pairs
+        k = k < n ? k : 0;
+        if (KEPT) return keep[k];
+        const float3 y = rel_pos(m, u, v0 + k);
+        return make_float4(y.x, y.y, y.z, 0.f);
+    };
     float best = 0.f;
     int row = 0;
     long long first = 0;  // index of the pair (row, row)
@@ -313,9 +327,9 @@ __global__ void __launch_bounds__(kExtentBlock) k_extent_pairs(const float4 *__r
         while (p >= first + nt - row) first += nt - row++;
         const int i = row * kExtentBlock + threadIdx.x, j = (row + (int)(p - first)) * kExtentBlock + threadIdx.x;
         __syncthreads();
-        tile[threadIdx.x] = keep[j < n ? j : 0];  // padding takes vertex 0: real pairs
+        tile[threadIdx.x] = at(j);
         __syncthreads();
-        const float4 q = keep[i < n ? i : 0];
+        const float4 q = at(i);
         const float3 y = make_float3(q.x, q.y, q.z);
 #pragma unroll 8
         for (int k = 0; k < kExtentBlock; ++k) {
@@ -328,12 +342,43 @@ __global__ void __launch_bounds__(kExtentBlock) k_extent_pairs(const float4 *__r
     if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(best));
 }
 
+// A cell of one tile: one block, its maximum stored without an atomic, so that
+// *out can be mapped host memory.
+__global__ void __launch_bounds__(kExtentBlock) k_extent_one(MeshView m, const float4 *__restrict__ u, int v0, int nv,
+                                                             unsigned *out) {
+    __shared__ float3 tile[kExtentBlock];
+    __shared__ float most[kExtentBlock / 32];
+    const float3 y = rel_pos(m, u, v0 + min((int)threadIdx.x, nv - 1));
+    tile[threadIdx.x] = y;
+    __syncthreads();
+    float best = 0.f;
+    for (int k = 0; k < nv; ++k) best = fmaxf(best, dist2(tile[k], y));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if ((threadIdx.x & 31) == 0) most[threadIdx.x >> 5] = best;
+    __syncthreads();
+    if (threadIdx.x > 0) return;
+    for (int w = 1; w < kExtentBlock / 32; ++w) best = fmaxf(best, most[w]);
+    *out = __float_as_uint(best);
+}
+
+cudaError_t launch_extent_one(const MeshView &m, const float4 *u, int v0, int nv, unsigned *out, cudaStream_t s) {
+    k_extent_one<<<1, kExtentBlock, 0, s>>>(m, u, v0, nv, out);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_max_extent(const MeshView &m, const float4 *u, int v0, int nv, float4 *keep, unsigned *out,
                               int blocks, cudaStream_t s) {
-    if (nv <= 0) return cudaMemsetAsync(out, 0, sizeof(unsigned), s);
+    const long long nt = (nv + kExtentBlock - 1) / kExtentBlock;
+    if (nt * (nt + 1) / 2 <= blocks) {
+        const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned), s);
+        if (e != cudaSuccess || nv <= 0) return e;
+        k_extent_pairs<false><<<(int)(nt * (nt + 1) / 2), kExtentBlock, 0, s>>>(nullptr, nullptr, m, u, v0, nv, out);
+        return cudaGetLastError();
+    }
     int *nkeep = reinterpret_cast<int *>(out + 1);
     k_extent_select<<<kSelectCluster, kSelectBlock, 0, s>>>(m, u, v0, nv, keep, nkeep, out);
-    k_extent_pairs<<<blocks, kExtentBlock, 0, s>>>(keep, nkeep, out);
+    k_extent_pairs<true><<<blocks, kExtentBlock, 0, s>>>(keep, nkeep, m, u, v0, nv, out);
     return cudaGetLastError();
 }
 

@@ -373,7 +373,10 @@ cudaError_t launch_energy(const MeshView &m, const float4 *u, int t0, int t1, do
 // theta1, theta2, theta3, volume. partial: 10 doubles per 256 tets.
 // Squared largest distance between two of the vertices [v0, v0 + nv) at
 // displacements u, as the bits of a float in out[0] (device; out[1] is
-// scratch, as are the nv entries of keep), with `blocks` blocks.
+// scratch, as are the nv entries of keep), with `blocks` blocks; of at most
+// kExtentOne vertices in *out (device or mapped).
+constexpr int kExtentOne = 256;
+cudaError_t launch_extent_one(const MeshView &m, const float4 *u, int v0, int nv, unsigned *out, cudaStream_t s);
 cudaError_t launch_max_extent(const MeshView &m, const float4 *u, int v0, int nv, float4 *keep, unsigned *out,
                               int blocks, cudaStream_t s);
 cudaError_t launch_taylor(const MeshView &m, const float4 *u, int t0, int t1, double *partial, double *out,
