@@ -401,8 +401,10 @@ cf_status cf_relax(cf_ctx *ctx, int32_t n, double dt, double damping, int32_t re
  * path[0], path[1]: thread blocks per cell with which steps and reverse steps
  * keep a cell's state on chip, 0 where they take launches of their own for
  * every step (three for a step); path[2]: steps of one launch on chip, at most
- * (a recorded call: one launch per checkpoint). The results of a step are the
- * same bits either way. CF_ESTATE without cells. */
+ * (a recorded call: one launch per checkpoint). Calls of one or two steps may
+ * take launches all the same, and so do the first steps on new cells (fewer
+ * than 32) unless this call came before them: it prepares the way on chip. The
+ * results of a step are the same bits either way. CF_ESTATE without cells. */
 #define CF_RELAX_PATH_LEN 3
 cf_status cf_get_relax_path(cf_ctx *ctx, int32_t *path);
 

@@ -146,10 +146,11 @@ struct cf_ctx {
     double *grad = nullptr, *gtmp = nullptr, *pforce = nullptr, *dF = nullptr;
     int adj_V = 0, adj_C = 0;
     // on-chip relaxation (csrc/relax.cu): the plan of the current mesh, made
-    // by the first relaxation; plan_state 0: not made, 1: made, 2: the mesh
+    // by the relaxation that brings its steps to kPlanSteps; plan_state 0: not made, 1: made, 2: the mesh
     // does not fit or is faster in launches. Given back where cells are added,
     // the lattice is allocated, or a checkpoint or a field finds no memory.
     int plan_state = 0;
+    long long plan_steps = 0;  // steps taken before the plan, up to kPlanSteps
     RelaxPlan plan{};
     RelaxPart *plan_parts = nullptr;
     float4 *plan_rows = nullptr;

@@ -485,7 +485,8 @@ struct RelaxPart {
 };
 struct RelaxPlan {
     int cs, nparts, NT;      // blocks per cell, parts, tets of all parts
-    bool steps, reverse;     // steps, reverse steps are taken on chip
+    int from;                // calls of that many steps or more are taken on chip (INT_MAX: none)
+    bool reverse;            // reverse steps are
     int per_tet;             // tets have material slots of their own (MeshView::tmat)
     size_t smem_step, smem_reverse;
     const RelaxPart *parts;  // [nparts], cs per cell

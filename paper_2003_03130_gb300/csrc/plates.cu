@@ -12,6 +12,7 @@
 //   lambda_y <- lambda_y + dt (J_el + J_plate) m, lambda_v <- c m,
 // accumulating dt m . df/d(mu, kappa, w) per cell in double.
 #include <algorithm>
+#include <cmath>
 #include <functional>
 #include <new>
 #include <queue>
@@ -22,6 +23,12 @@ namespace {
 
 constexpr int kTapeStride = 50;
 constexpr int kRelaxSteps = 1000;  // steps of one launch, at most (3 to 20 ms a wave of cells)
+// Steps in launches of their own before the on-chip plan is made, which takes
+// 60 us (a cell of 192 tets) to 350 (64 of 8.3 k) once per mesh: a mesh that is
+// relaxed by a few steps need not pay it (a first call of one step 24 to 82 us,
+// with the plan 80 to 440). A first call of 32 steps is at worst 8 % longer than
+// in launches (200 cells of 1.2 k tets: 705 and 655 us), one of 64 never.
+constexpr int kPlanSteps = 32;
 
 void free_adjoint(cf_ctx *c) {
     for (auto *p : c->ckpt) cudaFree(p);
@@ -44,6 +51,7 @@ void free_adjoint(cf_ctx *c) {
     dfree(c->zlo);
     dfree(c->zhi);
     cf_free_plan(c);
+    c->plan_steps = 0;
     c->adj_V = c->adj_C = 0;
 }
 
@@ -98,6 +106,10 @@ struct StepTime {
 };
 constexpr StepTime kChipStep{0.0, 2.15, 2.92e-3, 0.0}, kChipReverse{0.0, 4.9, 8.6e-3, 0.0};
 constexpr StepTime kLaunchStep{12.4, 10.9, 3.4e-5, 1.8e-5}, kLaunchReverse{25.0, 25.8, 5.9e-5, 1.47e-4};
+// A launch on chip takes 2 us more than its steps, and each wave of cells 4 (the
+// state of a cell, read and written): a call of one step of 8.3 k tets 20.9 us,
+// in launches 19.8.
+constexpr double kChipCall = 2.0, kChipWave = 4.0;
 
 double step_time(const StepTime &q, double nt, double nv) {
     return std::max(q.least, q.a + q.tet * nt + q.vertex * nv);
@@ -157,6 +169,8 @@ cudaError_t build_plan(cf_ctx *c) {
         cudaGetLastError();
         return cudaSuccess;
     }
+    for (const int4 &q : cells)  // some block of eight holds an eighth of a cell's tets or more
+        if (relax_smem(q.y, q.y, (q.w + 7) / 8, true) > (size_t)(smem - kRelaxStatic)) return cudaSuccess;
     const MeshView m = view(c);
     PlanScratch d;
 #define TRY_P(expr)                                \
@@ -211,9 +225,11 @@ cudaError_t build_plan(cf_ctx *c) {
     const int slots = relax_clusters(pl);
     if (slots == 0) return cudaSuccess;
     largest(cs, fits);
-    pl.steps = on_chip_time(kChipStep, most_of, slots) < step_time(kLaunchStep, c->T, c->V);
+    const double gain = step_time(kLaunchStep, c->T, c->V) - on_chip_time(kChipStep, most_of, slots);
+    const double call = kChipCall + kChipWave * ((C + slots - 1) / slots);
+    pl.from = gain > 0.0 ? (int)std::min(1e9, 1.0 + std::floor(call / gain)) : INT_MAX;
     pl.reverse = on_chip_time(kChipReverse, most_of, slots) < step_time(kLaunchReverse, c->T, c->V);
-    if (!pl.steps && !pl.reverse) return cudaSuccess;
+    if (pl.from == INT_MAX && !pl.reverse) return cudaSuccess;
     TRY_P(dalloc(&c->plan_parts, parts.size()));
     TRY_P(dalloc(&c->plan_rows, 3 * (size_t)pl.NT));
     TRY_P(dalloc(&c->plan_list, pl.NT));
@@ -254,10 +270,17 @@ cf_status make_plan(cf_ctx *c) {
                : fail(c, CF_ECUDA, "relaxation plan: %s", cudaGetErrorString(e));
 }
 
-// The plan if the mesh has one that takes steps (reverse: reverse steps) on
+// The plan before n more steps are taken, once enough of them are.
+cf_status plan_before(cf_ctx *c, long long n) {
+    if (c->plan_state) return CF_OK;
+    c->plan_steps = std::min(c->plan_steps + n, (long long)kPlanSteps);
+    return c->plan_steps < kPlanSteps ? CF_OK : make_plan(c);
+}
+
+// The plan if the mesh has one that takes n steps (reverse: n reverse steps) on
 // chip, with the materials' present form.
-const RelaxPlan *plan_of(cf_ctx *c, bool reverse) {
-    if (c->plan_state != 1 || !(reverse ? c->plan.reverse : c->plan.steps)) return nullptr;
+const RelaxPlan *plan_of(cf_ctx *c, bool reverse, int n) {
+    if (c->plan_state != 1 || !(reverse ? c->plan.reverse : n >= c->plan.from)) return nullptr;
     c->plan.per_tet = 0;
     for (const CellInfo &ci : c->cells) c->plan.per_tet |= ci.per_tet;
     return &c->plan;
@@ -351,9 +374,9 @@ cf_status cf_relax(cf_ctx *c, int32_t n, double dt, double damping, int32_t reco
             c->ckpt.push_back(p);
         }
     }
-    st = make_plan(c);
+    st = plan_before(c, n);
     if (st != CF_OK) return st;
-    const RelaxPlan *pl = plan_of(c, false);
+    const RelaxPlan *pl = plan_of(c, false, n);
     for (int k = 0; pl && k < n;) {  // on chip: a launch per checkpoint, or per kRelaxSteps
         const int b = std::min(record ? kTapeStride : kRelaxSteps, n - k);
         CUDA_TRY(c, launch_relax_cells(*pl, m, u, c->vel_r, u, c->vel_r,
@@ -386,8 +409,8 @@ cf_status cf_get_relax_path(cf_ctx *c, int32_t *path) {
     if (!path) return fail(c, CF_EINVAL, "null output");
     st = make_plan(c);
     if (st != CF_OK) return st;
-    path[0] = plan_of(c, false) ? c->plan.cs : 0;
-    path[1] = plan_of(c, true) ? c->plan.cs : 0;
+    path[0] = plan_of(c, false, kRelaxSteps) ? c->plan.cs : 0;
+    path[1] = plan_of(c, true, kRelaxSteps) ? c->plan.cs : 0;
     path[2] = kRelaxSteps;
     return CF_OK;
 }
@@ -438,9 +461,9 @@ cf_status cf_relax_adjoint(cf_ctx *c, const double *dF) {
     if (st != CF_OK) return st;
     CUDA_TRY(c, cudaMemcpyAsync(c->dF, dF, sizeof(double) * C, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, launch_adj_seed(m, c->ckpt[e.ck0 + e.nck - 1], e.kp, c->zlo, c->zhi, c->dF, c->lam, c->stream));
-    st = make_plan(c);
+    st = plan_before(c, 3LL * e.n);  // a step again and its reverse, which takes two
     if (st != CF_OK) return st;
-    const RelaxPlan *pl = plan_of(c, true);
+    const RelaxPlan *pl = plan_of(c, true, e.n);
     if (!pl) CUDA_TRY(c, launch_adj_m(c->V, c->lam, c->lamv, e.dt, c->mvec, c->stream));
     for (int j = e.nck - 2; j >= 0; --j) {
         const int s0 = j * kTapeStride, len = std::min(kTapeStride, e.n - s0);

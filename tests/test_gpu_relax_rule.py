@@ -66,3 +66,19 @@ def test_more_cells_than_slots_match_the_general_path(P, name):  # noqa: F811
         assert np.array_equal(x, y)
     # FP32 tangents summed in the same order: a few roundings (2^-24) a step
     assert np.linalg.norm(grads[0] - grads[1]) <= 1e-5 * np.linalg.norm(grads[1])
+
+
+@pytest.mark.parametrize("name", ["few", "two_waves"])
+def test_calls_of_few_steps_take_the_same_steps(P, name):  # noqa: F811
+    """The way on chip prepared beforehand, so that single steps take it, and left to the steps that make it worth it."""
+    got = []
+    for prepare in (True, False):
+        ctx = context(P, meshes(name), False, 8)
+        if prepare:
+            assert P.cf_get_relax_path(ctx)["step_blocks"] > 0
+        for n in (1, 1, 2, 27, 1, 40):
+            P.cf_relax(ctx, n, 0.02, 0.9)
+            got.append(P.cf_get_positions(ctx, P.CF_ALL_CELLS))
+        P.cf_destroy(ctx)
+    for a, b in zip(got[:6], got[6:]):
+        assert np.array_equal(a, b)
