@@ -164,20 +164,43 @@ void shape_to_lbm(LbmParams &p, const Shape &sh) {
     p.pairs = sh.pop_pairs;
 }
 
-// The lattice of a step of parity p: whether it is swept to and fro, and the
-// step's direction. With cells from both buffers larger than L2 (turn); a run
-// of the fluid alone (alone), whose data nothing else in L2 competes with,
-// from half of that, but not node pairs in rows that leave a third of a block
-// or more idle: issue bounds them there (csrc/lbm.cu has the figures).
-LbmParams sweep(const cf_ctx *c, int p, bool alone = false) {
-    LbmParams q = c->lp;
-    if (alone) {
-        const int pairs = q.nx / 2, block = std::min(pairs, 64);
-        const bool idle = pop_bytes(q.fmt) == 2 && q.pairs && q.nx % 2 == 0 &&
-                          3 * pairs < 2 * block * ((pairs + block - 1) / block);
-        q.turn = 2 * pop_bytes(q.fmt) * 19 * (size_t)q.N > (size_t)c->l2_bytes / 2 && !idle;
+// Whether a step's lattice is swept to and fro, its results kept in L2
+// (csrc/lbm.cu, KEEP, has the figures). A sweep finds at most an L2 of planes
+// from the one before, so both buffers together should exceed L2, beside which
+// nothing else has to fit there (half of it for the fluid alone), and not by
+// more than some 10 times (FP32 256^3 1 % slower with it, FP16 256^3 1 %
+// faster). The near field moves its populations, forces and velocities in
+// between: from a quarter of L2 on they have the planes evicted, and the kept
+// ones in turn the cells' data (16 cells of R = 8 in 128x190x200, 39 MB: 124.1
+// -> 122.0 us a step; in 222x190x114 151.4 -> 154.8; 60 cells there 223 -> 225,
+// in 130x120x110 110 -> 115). Node pairs in rows that leave a third of a block or
+// more idle are bound by issue and gain nothing (FP16 160^3 with a cell 80.5 ->
+// 81.3).
+bool swept(const cf_ctx *c) {
+    const LbmParams &p = c->lp;
+    const double pop = 19.0 * pop_bytes(p.fmt), both = 2.0 * pop * p.N, l2 = c->l2_bytes;
+    const int pairs = p.nx / 2, block = std::min(pairs, 64);
+    if (pop_bytes(p.fmt) == 2 && p.pairs && p.nx % 2 == 0 && 3 * pairs < 2 * block * ((pairs + block - 1) / block))
+        return false;
+    if (both > 10.0 * l2) return false;
+    if (c->cells.empty()) return both > 0.5 * l2;
+    // nodes of the tiles about the cells' reference boxes
+    const double n[3] = {(double)p.nx, (double)p.ny, (double)p.nz};
+    const int shift[3] = {p.tlx, p.tly, p.tlz};
+    double near = 0.0;
+    for (const CellInfo &ci : c->cells) {
+        double box = 1.0;
+        for (int a = 0; a < 3; ++a) box *= std::min(n[a], ci.extent[a] + p.dw + 2.0 + (1 << shift[a]));
+        near += box;
     }
-    q.back = q.turn && p;
+    return both > l2 && near * (2.0 * pop + 32.0) < 0.25 * l2;
+}
+
+// The lattice of a step of parity p.
+LbmParams sweep(const cf_ctx *c, int p, bool turn) {
+    LbmParams q = c->lp;
+    q.turn = turn;
+    q.back = turn && p;
     return q;
 }
 
@@ -201,10 +224,11 @@ cf_status enqueue_steps(cf_ctx *c, Kind kind, int p0, int s0, int nsteps, cudaSt
                                          RegionSlot{nullptr}, sh.interp_form));
         return CF_OK;
     }
+    const bool turn = swept(c);
     if (kind == Kind::Fluid) {
         for (int i = 0; i < nsteps; ++i) {
             const int p = p0 ^ (i & 1);
-            CUDA_TRY(c, launch_lbm(c->f[p], c->f[1 - p], sweep(c, p, true), c->seed + p, c->seed + 1 - p, sf));
+            CUDA_TRY(c, launch_lbm(c->f[p], c->f[1 - p], sweep(c, p, turn), c->seed + p, c->seed + 1 - p, sf));
         }
         return CF_OK;
     }
@@ -223,7 +247,7 @@ cf_status enqueue_steps(cf_ctx *c, Kind kind, int p0, int s0, int nsteps, cudaSt
         const int p = p0 ^ (i & 1), s = (s0 + i) % 3;
         const RegionSlot use = region_slot(c, s), acc = accum_slot(c, s);
         if (i > 0) CUDA_TRY(c, cudaStreamWaitEvent(sf, ev_near[i - 1], 0));
-        CUDA_TRY(c, launch_lbm_far(c->f[p], c->f[1 - p], sweep(c, p), use.bits, c->seed + p, sh.far_spec, sf));
+        CUDA_TRY(c, launch_lbm_far(c->f[p], c->f[1 - p], sweep(c, p, turn), use.bits, c->seed + p, sh.far_spec, sf));
         CUDA_TRY(c, cudaEventRecord(ev_far[i], sf));
         if (!(first && i == 0)) {  // K5 of the previous step (parity 1-p), with mark_k5 marking acc
             CUDA_TRY(c, launch_interp_advect(m, c->vel, c->lp, c->u[1 - p], c->u[p], c->d_err, sc, sh.interp_block,
@@ -232,7 +256,7 @@ cf_status enqueue_steps(cf_ctx *c, Kind kind, int p0, int s0, int nsteps, cudaSt
         if (first && i == 0 && !sh.mark_k5) CUDA_TRY(c, clear_slot(c, acc, sc));
         CUDA_TRY(c, launch_chain_step(c, m, p, sh, acc, sc));
         if (i > 0) CUDA_TRY(c, cudaStreamWaitEvent(sc, ev_far[i - 1], 0));
-        CUDA_TRY(c, launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c, p), use.bits, c->vel,
+        CUDA_TRY(c, launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c, p, turn), use.bits, c->vel,
                                     sh.near_rows || !c->near_tiles_fit ? 0 : near_grid(c), c->seed + p, c->seed + 1 - p, next_slot(c, s).bits, sc));
         CUDA_TRY(c, cudaEventRecord(ev_near[i], sc));
     }
@@ -509,7 +533,6 @@ cf_status cf_lbm_init(cf_ctx *c, int32_t nx, int32_t ny, int32_t nz, double tau,
     }
     shape_to_lbm(p, c->shape);
     cudaDeviceGetAttribute(&c->l2_bytes, cudaDevAttrL2CacheSize, c->device);
-    p.turn = 2 * 19 * (long long)pop_bytes(p.fmt) * N > (long long)c->l2_bytes;  // both buffers
     c->region_bits_max = (tmax + 31) / 32;
     c->region_stride = (c->region_bits_max + 31) / 32 * 32;
     int smem_optin = 0;
@@ -577,12 +600,16 @@ cf_status cf_mesh_init_batch(cf_ctx *c, int32_t ncells, const int32_t *nv, const
     if (c->T + toff[ncells] > INT_MAX / 4 || c->V + voff[ncells] > INT_MAX / 4)
         return fail(c, CF_EINVAL, "mesh too large");
     for (int k = 0; k < ncells; ++k) {
-        double mean[3] = {0, 0, 0};
+        double mean[3] = {0, 0, 0}, lo[3], hi[3];
+        for (int a = 0; a < 3; ++a) lo[a] = hi[a] = x_ref[3 * voff[k] + a];
         for (long long v = voff[k]; v < voff[k + 1]; ++v)
             for (int a = 0; a < 3; ++a) {
-                if (!std::isfinite(x_ref[3 * v + a]) || (y0 && !std::isfinite(y0[3 * v + a])))
+                const double q = x_ref[3 * v + a];
+                if (!std::isfinite(q) || (y0 && !std::isfinite(y0[3 * v + a])))
                     return fail(c, CF_EINVAL, "cell %d: non-finite coordinate at vertex %lld", k, v - voff[k]);
-                mean[a] += x_ref[3 * v + a];
+                mean[a] += q;
+                lo[a] = std::min(lo[a], q);
+                hi[a] = std::max(hi[a], q);
             }
         CellInfo &ci = add[k];
         ci.v_off = c->V + (int)voff[k];
@@ -590,6 +617,7 @@ cf_status cf_mesh_init_batch(cf_ctx *c, int32_t ncells, const int32_t *nv, const
         ci.t_off = c->T + (int)toff[k];
         ci.nt = nt[k];
         for (int a = 0; a < 3; ++a) ci.origin[a] = (int)std::lround(mean[a] / nv[k]);
+        for (int a = 0; a < 3; ++a) ci.extent[a] = (float)(hi[a] - lo[a]);
         ci.mat = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     const int Vadd = (int)voff[ncells], Tadd = (int)toff[ncells];
@@ -959,7 +987,7 @@ cf_status timed_steps(cf_ctx *c, int n, const Shape &sh, double acc[5]) {
     for (int k = 0; k < 5; ++k) acc[k] = 0.0;
     cf_status st = CF_OK;
     const MeshView m = view(c);
-    const bool cells = c->T > 0;
+    const bool cells = c->T > 0, turn = swept(c);
     cudaStream_t s = c->stream;
     if (n > 0) c->macro_tile = cells ? sh.tile : -1;
     for (int done = 0; done < n && st == CF_OK;) {
@@ -992,11 +1020,11 @@ cf_status timed_steps(cf_ctx *c, int n, const Shape &sh, double acc[5]) {
                 e = launch_gather_spread(m, c->u[p], c->F, &c->lp, c->d_err, s, sh.gather_block, sh.staged);
             cudaEventRecord(E[3], s);
             if (e == cudaSuccess)
-                e = cells ? launch_lbm_far(c->f[p], c->f[1 - p], sweep(c, p), use.bits, c->seed + p, sh.far_spec, s)
-                          : launch_lbm(c->f[p], c->f[1 - p], sweep(c, p, true), c->seed + p, c->seed + 1 - p, s);
+                e = cells ? launch_lbm_far(c->f[p], c->f[1 - p], sweep(c, p, turn), use.bits, c->seed + p, sh.far_spec, s)
+                          : launch_lbm(c->f[p], c->f[1 - p], sweep(c, p, turn), c->seed + p, c->seed + 1 - p, s);
             cudaEventRecord(E[4], s);
             if (cells && e == cudaSuccess)
-                e = launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c, p), use.bits, c->vel,
+                e = launch_lbm_near(c->f[p], c->f[1 - p], c->F, sweep(c, p, turn), use.bits, c->vel,
                                     sh.near_rows || !c->near_tiles_fit ? 0 : near_grid(c), c->seed + p, c->seed + 1 - p,
                                     next_slot(c, sph).bits, s);
             cudaEventRecord(E[5], s);

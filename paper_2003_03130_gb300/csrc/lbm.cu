@@ -17,11 +17,10 @@
 // FP16 / BF16 multiplied by a power of two per weight class (2^14, 2^16, 2^17
 // for w = 1/3, 1/18, 1/36, so that the stored values are O(10^3) and never
 // subnormal in FP16); the collide always runs in FP32. Population loads
-// carry the streaming cache hint (evict first), and so do the stores of a
-// lattice that fits L2 beside cells: every population is touched once per
-// step, and the hint keeps the cells' few MB of mesh data resident in L2 while
-// the lattice streams through it. Other lattices are swept to and fro and keep
-// their results (KEEP below).
+// carry the streaming cache hint (evict first), and so do the stores but where
+// the lattice is swept to and fro (KEEP below): every population is touched once
+// per step, and the hint keeps the cells' few MB of mesh data resident in L2
+// while the lattice streams through it.
 //
 // One node per thread: 19 independent coalesced loads per node (x-shifted
 // rows are off by one word; neighbouring warps share the lines in L2), the
@@ -56,10 +55,11 @@ namespace cf {
 // both buffers (FP32 80^3 12.2 -> 11.8 us a step, 96^3 20.4 -> 17.4, 128^3
 // 50.1 -> 45.5, 192^3 163.7 -> 159.8; FP16 104^3 17.2 -> 16.6, 128^3 27.5 ->
 // 25.6), smaller ones nothing, nor node pairs in half-empty blocks (FP16 160^3
-// 71.2 -> 72.0). With cells it is worth it once both buffers exceed L2 (128^3
-// with a cell, FP32 52.4 -> 48.2, FP16 31.4 -> 29.5; FP16 160^3 78.0 -> 77.2);
-// in a lattice that fits, the kept results evict the cells' data (512x64x40
-// FP16 with a cell 21.2 -> 22.0, 80x128x64 FP32 with 8 cells 41.8 -> 43.6).
+// 71.2 -> 72.0). With few cells it is worth it once both buffers exceed L2
+// (128^3 with a cell, FP32 52.4 -> 48.2, FP16 31.4 -> 29.5); in a lattice that
+// fits, the kept results evict the cells' data (512x64x40 FP16 with a cell 21.2
+// -> 22.0, 80x128x64 FP32 with 8 cells 41.8 -> 43.6). Very large lattices and
+// those with many cells lose (figures at the rule, `swept` in capi.cu).
 // KEEP is a template argument: a policy operand on each store cost a 16-bit
 // step 1 to 2 % and 32^3 FP32 7 %, a branch around the stores the node pairs
 // up to 4 %, and a lattice that is not swept needs none of it.
