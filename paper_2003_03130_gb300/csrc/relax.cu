@@ -23,15 +23,17 @@
 // blocks a cluster, 65,535 vertices a cell and 32 incidences a vertex) and
 // where it is expected to be faster (csrc/plates.cu, make_plan).
 //
-// Bound by instruction issue (0.6 of the slots: ~400 instructions a tet, ~40
-// an incidence). 64 cells of 8.3 k tets (1,853 vertices) on 128 SMs: 17.5 us a
-// step, where the three launches took 29 (the corner forces cross L2 there, 64
-// bytes written and read per tet); a reverse step 30 us, 53 before. Two cells
-// of 1.2 k tets: 5 to 6 us a step of either kind, 15 and 25 before. Velocities
-// stay in shared memory and the trail is stored a step late, since a barrier's
-// release waits for every store still on its way (19 -> 17.5 us). Measured and
-// not taken: every tet in one block only, corner forces read from the
-// neighbour through distributed shared memory (20.5 us).
+// Bound by instruction issue and the two barriers of a step: 655 warp
+// instructions per 32 tets, incidences included, in 0.71 of the slots of the SMs
+// that have a block (reverse steps 1,040 in 0.62). 64 cells of 8.3 k tets (1,863
+// vertices) on 128 SMs: 16.2 us a step, where three launches take 29 (the corner
+// forces cross L2 there, 64 bytes written and read per tet); a reverse step
+// 30.5 us, 40 in launches. A cell of 1.2 k tets: 3.2 us a step and 4.6 a reverse
+// one, 12.4 and 14 in launches. Velocities stay in shared memory and the trail is
+// stored a step late, since a barrier's release waits for every store still on
+// its way (19 -> 17.5 us). Measured and not taken: every tet in one block only,
+// corner forces read from the neighbour through distributed shared memory (20.5
+// us).
 #include <climits>
 
 #include "cell_ops.cuh"
