@@ -600,16 +600,12 @@ cf_status cf_mesh_init_batch(cf_ctx *c, int32_t ncells, const int32_t *nv, const
     if (c->T + toff[ncells] > INT_MAX / 4 || c->V + voff[ncells] > INT_MAX / 4)
         return fail(c, CF_EINVAL, "mesh too large");
     for (int k = 0; k < ncells; ++k) {
-        double mean[3] = {0, 0, 0}, lo[3], hi[3];
-        for (int a = 0; a < 3; ++a) lo[a] = hi[a] = x_ref[3 * voff[k] + a];
+        double mean[3] = {0, 0, 0};
         for (long long v = voff[k]; v < voff[k + 1]; ++v)
             for (int a = 0; a < 3; ++a) {
-                const double q = x_ref[3 * v + a];
-                if (!std::isfinite(q) || (y0 && !std::isfinite(y0[3 * v + a])))
+                if (!std::isfinite(x_ref[3 * v + a]) || (y0 && !std::isfinite(y0[3 * v + a])))
                     return fail(c, CF_EINVAL, "cell %d: non-finite coordinate at vertex %lld", k, v - voff[k]);
-                mean[a] += q;
-                lo[a] = std::min(lo[a], q);
-                hi[a] = std::max(hi[a], q);
+                mean[a] += x_ref[3 * v + a];
             }
         CellInfo &ci = add[k];
         ci.v_off = c->V + (int)voff[k];
@@ -617,7 +613,14 @@ cf_status cf_mesh_init_batch(cf_ctx *c, int32_t ncells, const int32_t *nv, const
         ci.t_off = c->T + (int)toff[k];
         ci.nt = nt[k];
         for (int a = 0; a < 3; ++a) ci.origin[a] = (int)std::lround(mean[a] / nv[k]);
-        for (int a = 0; a < 3; ++a) ci.extent[a] = (float)(hi[a] - lo[a]);
+        for (int a = 0; a < 3; ++a) {  // of some 500 vertices: an estimate of the near field's size needs no more
+            double lo = x_ref[3 * voff[k] + a], hi = lo;
+            for (long long v = voff[k]; v < voff[k + 1]; v += nv[k] / 512 + 1) {
+                lo = std::min(lo, x_ref[3 * v + a]);
+                hi = std::max(hi, x_ref[3 * v + a]);
+            }
+            ci.extent[a] = (float)(hi - lo);
+        }
         ci.mat = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     const int Vadd = (int)voff[ncells], Tadd = (int)toff[ncells];

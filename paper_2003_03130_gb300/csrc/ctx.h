@@ -25,7 +25,7 @@ struct CellInfo {
     int origin[3];
     float4 mat;
     bool per_tet = false;  // tets carry their own material slots (cf_set_tet_materials)
-    float extent[3];  // of the reference positions
+    float extent[3];  // of the reference positions, about
 };
 
 // Force-region tile shapes (log2 of the x, y, z extents; 256 nodes each).
