@@ -30,9 +30,12 @@ def cells(P, n, general=False):  # noqa: F811
 def fill(leave):
     """Tensors that take the device's free memory but for `leave` bytes."""
     torch.cuda.empty_cache()
-    held = [torch.empty(torch.cuda.mem_get_info(0)[0] - leave - 64 * MB, dtype=torch.uint8, device="cuda:0")]
-    while torch.cuda.mem_get_info(0)[0] > leave + 4 * MB:
-        held.append(torch.empty(torch.cuda.mem_get_info(0)[0] - leave - 2 * MB, dtype=torch.uint8, device="cuda:0"))
+    try:
+        held = [torch.empty(torch.cuda.mem_get_info(0)[0] - leave - 64 * MB, dtype=torch.uint8, device="cuda:0")]
+        while torch.cuda.mem_get_info(0)[0] > leave + 4 * MB:
+            held.append(torch.empty(torch.cuda.mem_get_info(0)[0] - leave - 2 * MB, dtype=torch.uint8, device="cuda:0"))
+    except torch.cuda.OutOfMemoryError:
+        pytest.skip("the device's free memory is in use elsewhere")
     return held
 
 
